@@ -87,12 +87,7 @@ __device__ __forceinline__ int solve_face(const SegCtx<T> &s, int D, const T *qa
     qL[v] = qa[v * qs] + T(0.5) * qa[(5 + 5 * D + v) * qs];
     qR[v] = qb[v * qs] - T(0.5) * qb[(5 + 5 * D + v) * qs];
   }
-  if (D == 0)
-    face_flux_states<0>(s, qL, qR, F);
-  else if (D == 1)
-    face_flux_states<1>(s, qL, qR, F);
-  else
-    face_flux_states<2>(s, qL, qR, F);
+  face_flux_states(D, s, qL, qR, F);
   if ((ta == kCellGhost) == (tb == kCellGhost)) return 2;
   return tb == kCellGhost ? 1 : -1;
 }
@@ -198,16 +193,6 @@ __device__ __forceinline__ int face_kind(uint8_t ta_full, uint8_t tb_full) {
   if (!(ta != kCellNone && tb != kCellNone && ta != kCellSplit && tb != kCellSplit && own_leaf)) return 0;
   if ((ta == kCellGhost) == (tb == kCellGhost)) return 2;
   return tb == kCellGhost ? 1 : -1;
-}
-
-template <class T>
-__device__ __forceinline__ void face_flux_dir(const SegCtx<T> &s, int D, T (&qL)[5], T (&qR)[5], T (&F)[5]) {
-  if (D == 0)
-    face_flux_states<0>(s, qL, qR, F);
-  else if (D == 1)
-    face_flux_states<1>(s, qL, qR, F);
-  else
-    face_flux_states<2>(s, qL, qR, F);
 }
 
 template <class T, int NS>
@@ -415,7 +400,7 @@ __global__ void __launch_bounds__(Rock<NS>::THREADS, Rock<NS>::template min_bloc
 #pragma unroll
           for (int v = 0; v < 5; ++v) qR[v] = sQ[v * IC + gp] - T(0.5) * sQ[(5 + 5 * D + v) * IC + gp];
         }
-        face_flux_dir(s, D, qL, qR, F);
+        face_flux_states(D, s, qL, qR, F);
         if (a.reflux && (kind == 1 || kind == -1)) {
           const int cg = kind > 0 ? cb : ca;
           const int gx = cg % E, gy = (cg / E) % E, gz = cg / (E * E);
