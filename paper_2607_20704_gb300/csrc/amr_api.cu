@@ -888,7 +888,7 @@ static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double d
   } else {
     // FP64: every predictor and every face solve exactly once
     run_list(h, K_PRIM, k_prim<T>, a, L, DOM_CELLS);
-    run_list(h, K_PREDICT, k_predict<T>, a, L, DOM_CELLS);
+    run_list(h, K_PREDICT, k_predict, a, L, DOM_CELLS);
     run_list(h, K_FLUX, k_flux<T>, a, L, DOM_CELLS);
     run_list(h, K_UPDATE, k_update<T>, a, L, DOM_REAL);
   }
@@ -1064,11 +1064,12 @@ static void destroy_all(amr_mesh *h) {
 
 template <class T>
 static amr_status upload_member_params(amr_mesh *h) {
-  std::vector<T> g(h->M), igm1(h->M), sr(h->M), sp(h->M);
+  std::vector<T> g(h->M), igm1(2 * size_t(h->M)), sr(h->M), sp(h->M);
   for (int q = 0; q < h->M; ++q) {
     const Member &m = h->mem[q];
     g[q] = T(m.gamma);
-    igm1[q] = T(1.0 / (m.gamma - 1.0));
+    igm1[2 * size_t(q)] = T(1.0 / (m.gamma - 1.0));
+    igm1[2 * size_t(q) + 1] = g[q] - T(1);
     sr[q] = T(m.smallr);
     sp[q] = T(m.smallc * m.smallc / m.gamma);
   }

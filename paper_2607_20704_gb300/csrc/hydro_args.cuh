@@ -67,7 +67,7 @@ struct StepArgs {
   const Seg *segs;
   const int *tpre;                  // the list's tile prefix (see Tile)
   int tseg0, tnseg, tstep, ntiles;  // first segment, segments, items per tile, tiles
-  // per member: gamma, 1/(gamma-1), floors
+  // per member: gamma, {1/(gamma-1), gamma-1}, floors
   const T *mgamma, *migm1, *msmallr, *msmallp;
   // dt/dx: from the device time step of each member's coarse step
   // (dt_m 2^levelmin_m, the same for every level of the member), or, when

@@ -119,7 +119,7 @@ __device__ __forceinline__ float sound_speed(float c2) { return sqrtf(c2); }
 template <class T>
 struct SegCtx {
   int lo, nl, clo, ncl, base, flags;
-  T gamma, igm1, smallr, smallp, dtdx;
+  T gamma, gm1, igm1, smallr, smallp, dtdx;  // gm1 = gamma - 1, igm1 = 1 / gm1
 };
 
 __device__ __forceinline__ double seg_dtdx(const StepArgs<double> &a, const Seg &s) {
@@ -141,7 +141,8 @@ __device__ __forceinline__ SegCtx<T> seg_ctx(const StepArgs<T> &a, int seg) {
   c.base = s.base;
   c.flags = s.flags;
   c.gamma = __ldg(a.mgamma + s.member);
-  c.igm1 = __ldg(a.migm1 + s.member);
+  c.igm1 = __ldg(a.migm1 + 2 * s.member);
+  c.gm1 = __ldg(a.migm1 + 2 * s.member + 1);
   c.smallr = __ldg(a.msmallr + s.member);
   c.smallp = __ldg(a.msmallp + s.member);
   c.dtdx = seg_dtdx(a, s);
@@ -230,19 +231,69 @@ __global__ void k_prolong(StepArgs<T> a) {
 // ---------------------------------------------------------------------------
 // primitives of every real and ghost cell; domain: 8 (nl + ncl)
 // ---------------------------------------------------------------------------
+// The plain products of the FP64 arithmetic: every operation rounded as written,
+// so that a result has the same bits in every kernel, on the FP64 pipe (MulFp64)
+// or on the integer pipes (MulInt), which are otherwise idle.  mul0 is for operands that can be
+// tiny or zero (a product below the normal range is zero in both).
+struct MulFp64 {
+  static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+  static __device__ __forceinline__ double mul0(double a, double b) { return mul_fp64_0(a, b); }
+  static __device__ __forceinline__ double half(double a) { return __dmul_rn(0.5, a); }
+};
+struct MulInt {
+  static __device__ __forceinline__ double mul(double a, double b) { return mul_int(a, b); }
+  static __device__ __forceinline__ double mul0(double a, double b) { return mul_int0(a, b); }
+  static __device__ __forceinline__ double half(double a) {  // exponent - 1
+    return __hiloint2double(__double2hiint(a) - (1 << 20), __double2loint(a));
+  }
+};
+
+// p <- max(p, r smallp), r > 0.  FP64: when p's exponent lies two above that
+// of r smallp the floor cannot act, and its product is not formed
+__device__ __forceinline__ float floor_p(float p, float r, float smallp) { return vmax(p, r * smallp); }
+__device__ __forceinline__ double floor_p(double p, double r, double smallp) {
+  if (__double2hiint(p) <= __double2hiint(r) + (__double2hiint(smallp) - (1021 << 20))) p = vmax(p, r * smallp);
+  return p;
+}
+
 // primitives (rho, u, v, w, p) of the conservative state (u0..u4), with the
 // density and pressure floors
-template <class T>
-__device__ __forceinline__ void prim_of(const SegCtx<T> &s, T u0, T u1, T u2, T u3, T u4, T (&w)[5]) {
-  const T r = vmax(u0, s.smallr);
-  const T ir = rcp(r);
-  const T vx = u1 * ir, vy = u2 * ir, vz = u3 * ir;
-  const T ek = T(0.5) * r * ((vx * vx + vy * vy) + vz * vz);
+__device__ __forceinline__ void prim_of(const SegCtx<float> &s, float u0, float u1, float u2, float u3, float u4,
+                                        float (&w)[5]) {
+  const float r = vmax(u0, s.smallr);
+  const float ir = rcp(r);
+  const float vx = u1 * ir, vy = u2 * ir, vz = u3 * ir;
+  const float ek = 0.5f * r * ((vx * vx + vy * vy) + vz * vz);
   w[0] = r;
   w[1] = vx;
   w[2] = vy;
   w[3] = vz;
-  w[4] = vmax((s.gamma - T(1)) * (u4 - ek), r * s.smallp);
+  w[4] = vmax(s.gm1 * (u4 - ek), r * s.smallp);
+}
+template <class O>
+__device__ __forceinline__ void prim_fp64(const SegCtx<double> &s, double r, double u1, double u2, double u3,
+                                          double u4, double (&w)[5]) {
+  const double ir = rcp(r);
+  const double vx = O::mul0(u1, ir), vy = O::mul0(u2, ir), vz = O::mul0(u3, ir);
+  const double ek = O::mul0(O::half(r), __fma_rn(vz, vz, __fma_rn(vy, vy, O::mul0(vx, vx))));
+  w[0] = r;
+  w[1] = vx;
+  w[2] = vy;
+  w[3] = vz;
+  w[4] = floor_p(O::mul0(s.gm1, __dadd_rn(u4, -ek)), r, s.smallp);
+}
+// FP64: 6 of 12 operations are products that the integer pipes take when the
+// warp's densities lie in [2^-100, 2^100), momenta below 2^150 and energies
+// below 2^300 (nothing overflows then); 14 on the FP64 pipe otherwise
+__device__ __forceinline__ void prim_of(const SegCtx<double> &s, double u0, double u1, double u2, double u3,
+                                        double u4, double (&w)[5]) {
+  const double r = vmax(u0, s.smallr);
+  const bool safe = within<100>(r) && below<150>(u1) && below<150>(u2) && below<150>(u3) && below<300>(u4) &&
+                    within<100>(s.gm1);
+  if (__all_sync(__activemask(), safe))
+    prim_fp64<MulInt>(s, r, u1, u2, u3, u4, w);
+  else
+    prim_fp64<MulFp64>(s, r, u1, u2, u3, u4, w);
 }
 
 template <class T>
@@ -267,13 +318,12 @@ __global__ void k_prim(StepArgs<T> a) {
 // ---------------------------------------------------------------------------
 // limited slopes and Hancock predictor W* = W + dt/(2dx) S(W, dW)
 // ---------------------------------------------------------------------------
-template <class T>
-__device__ __forceinline__ void predictor(const SegCtx<T> &s, const T (&w)[5],
-                                          const T (&dw)[3][5], T (&ws)[5]) {
-  const T r = w[0], p = w[4], g = s.gamma;
-  const T ir = rcp(r);
-  const T gp = g * p;
-  T src[5];
+__device__ __forceinline__ void predictor(const SegCtx<float> &s, const float (&w)[5], const float (&dw)[3][5],
+                                          float (&ws)[5]) {
+  const float r = w[0], p = w[4], g = s.gamma;
+  const float ir = rcp(r);
+  const float gp = g * p;
+  float src[5];
   src[0] = -(((w[1] * dw[0][0] + r * dw[0][1]) + (w[2] * dw[1][0] + r * dw[1][2])) +
              (w[3] * dw[2][0] + r * dw[2][3]));
 #pragma unroll
@@ -282,9 +332,41 @@ __device__ __forceinline__ void predictor(const SegCtx<T> &s, const T (&w)[5],
         -((w[1] * dw[0][1 + k] + w[2] * dw[1][1 + k]) + w[3] * dw[2][1 + k]) - dw[k][4] * ir;
   src[4] = -(((w[1] * dw[0][4] + gp * dw[0][1]) + (w[2] * dw[1][4] + gp * dw[1][2])) +
              (w[3] * dw[2][4] + gp * dw[2][3]));
-  const T hdt = T(0.5) * s.dtdx;
+  const float hdt = 0.5f * s.dtdx;
 #pragma unroll
   for (int v = 0; v < 5; ++v) ws[v] = w[v] + hdt * src[v];
+}
+// FP64: the velocity divergence is formed once for the density and the
+// pressure, and each source is one chain of FMAs: 31 operations (42 with the
+// terms of each direction on their own), 6 of them products for the integer
+// pipes
+template <class O>
+__device__ __forceinline__ void predictor_fp64(const SegCtx<double> &s, const double (&w)[5],
+                                               const double (&dw)[3][5], double (&ws)[5]) {
+  const double ir = rcp(w[0]), gp = O::mul(s.gamma, w[4]);
+  const double div = __dadd_rn(__dadd_rn(dw[0][1], dw[1][2]), dw[2][3]);
+  const int hd = __double2hiint(s.dtdx);  // -dt/(2dx): exponent - 1, on the integer pipe
+  const double mh = (hd & 0x7FF00000) > (1 << 20)
+                        ? __hiloint2double(int(uint32_t(hd - (1 << 20)) ^ 0x80000000u), __double2loint(s.dtdx))
+                        : -0.5 * s.dtdx;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const double adv = __fma_rn(w[3], dw[2][v], __fma_rn(w[2], dw[1][v], O::mul0(w[1], dw[0][v])));
+    const double src = v == 0   ? __fma_rn(w[0], div, adv)
+                       : v == 4 ? __fma_rn(gp, div, adv)
+                                : __fma_rn(dw[v < 1 || v > 3 ? 0 : v - 1][4], ir, adv);
+    ws[v] = __fma_rn(mh, src, w[v]);
+  }
+}
+__device__ __forceinline__ void predictor(const SegCtx<double> &s, const double (&w)[5], const double (&dw)[3][5],
+                                          double (&ws)[5]) {
+  bool safe = within<100>(w[0]) && within<100>(w[4]) && below<150>(w[1]) && within<100>(s.gamma);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) safe = safe && below<300>(dw[0][v]);
+  if (__all_sync(__activemask(), safe))
+    predictor_fp64<MulInt>(s, w, dw, ws);
+  else
+    predictor_fp64<MulFp64>(s, w, dw, ws);
 }
 
 template <class T>
@@ -298,34 +380,65 @@ __device__ __forceinline__ void store_q(const StepArgs<T> &a, int o, const T (&w
     for (int v = 0; v < 5; ++v) a.Q[(5 + 5 * d + v) * a.LS + o] = dw[d][v];
 }
 
-template <class T>
-__global__ void k_predict(StepArgs<T> a) {
-  tile_loop(a, [](const SegCtx<T> &s) { return 8 * (s.nl + s.ncl); },
-            [&](const SegCtx<T> &s, int t) {
-              const int e = ext_of_local(a, s, t >> 3);
-              const int c = t & 7;
-              const int o = s.base + t;
-              T w[5], dw[3][5], ws[5];
+// FP64: one thread per cell, an oct in 8 neighbouring lanes.  Along each axis a
+// cell has one neighbour inside its oct and one outside; the inner difference
+// is the same number for both cells of a pair, so the pair's lanes each form it
+// for half of the variables and exchange it (24 differences per cell instead
+// of 30, and 15 loads instead of 30).  Bound by the FP64 pipe: 49 operations
+// per cell, 72 with every difference and product on it.
+__device__ __forceinline__ double shfl_xor_f64(unsigned mask, double x, int lanes) {
+  const int lo = __shfl_xor_sync(mask, __double2loint(x), lanes), hi = __shfl_xor_sync(mask, __double2hiint(x), lanes);
+  return __hiloint2double(hi, lo);
+}
+__global__ void k_predict(StepArgs<double> a) {
+  for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tpre, a.tseg0, a.tnseg, a.tstep, ti);
+    if (a.mact && !__ldg(a.mact + a.segs[td.seg].member)) continue;  // finished member
+    const SegCtx<double> s = seg_ctx(a, td.seg);
+#ifdef AMR_CHECKED
+    if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
+      atomicOr(a.err, kErrIndex);
+      continue;
+    }
+#endif
+    const int t = td.start + threadIdx.x;  // tiles start at multiples of 8: octs are whole
+    const bool on = t < 8 * (s.nl + s.ncl);
+    const unsigned lanes = __ballot_sync(0xFFFFFFFFu, on);
+    if (!on) continue;
+    const int e = ext_of_local(a, s, t >> 3);
+    const int c = t & 7;
+    const int o = s.base + t;
+    double w[5], dw[3][5], ws[5];
 #pragma unroll
-              for (int v = 0; v < 5; ++v) w[v] = a.W[v * a.LS + o];
+    for (int v = 0; v < 5; ++v) w[v] = a.W[v * a.LS + o];
 #pragma unroll
-              for (int d = 0; d < 3; ++d) {
-                const int tm = nbr_local(a, s, t, e, c, d, 0);
-                const int tp = nbr_local(a, s, t, e, c, d, 1);
-                if (tm < 0 || tp < 0) {  // outer ring of a ghost oct: never used
+    for (int d = 0; d < 3; ++d) {
+      const int bit = 1 << d;
+      const bool up = c & bit;  // the pair's cell on the plus side
+      double in[5];             // inner differences, plus side minus minus side
 #pragma unroll
-                  for (int v = 0; v < 5; ++v) dw[d][v] = T(0);
-                  continue;
-                }
+      for (int v = 0; v < 4; v += 2) {  // the minus side's lane forms v, the plus side's v + 1
+        const double got = shfl_xor_f64(lanes, up ? w[v] : w[v + 1], bit);
+        const double mine = (up ? w[v + 1] : got) - (up ? got : w[v]);
+        const double other = shfl_xor_f64(lanes, mine, bit);
+        in[v] = up ? other : mine;
+        in[v + 1] = up ? mine : other;
+      }
+      const double got = shfl_xor_f64(lanes, w[4], bit);
+      in[4] = (up ? w[4] : got) - (up ? got : w[4]);
+      const int to = nbr_local(a, s, t, e, c, d, up ? 1 : 0);
 #pragma unroll
-                for (int v = 0; v < 5; ++v) {
-                  const T wm = a.W[v * a.LS + s.base + tm], wp = a.W[v * a.LS + s.base + tp];
-                  dw[d][v] = minmod(wp - w[v], w[v] - wm);
-                }
-              }
-              predictor(s, w, dw, ws);
-              store_q(a, o, ws, dw);
-            });
+      for (int v = 0; v < 5; ++v) {
+        dw[d][v] = 0.0;  // outer ring of a ghost oct: never used
+        if (to >= 0) {
+          const double wo = a.W[v * a.LS + s.base + to];
+          dw[d][v] = minmod((up ? wo : w[v]) - (up ? w[v] : wo), in[v]);
+        }
+      }
+    }
+    predictor(s, w, dw, ws);
+    store_q(a, o, ws, dw);
+  }
 }
 
 // FP32: primitives of the cell and its six face neighbours derived from U
@@ -357,23 +470,6 @@ __global__ void __launch_bounds__(512, 3) k_predict_u(StepArgs<T> a) {
               store_q(a, s.base + t, ws, dw);
             });
 }
-
-// The plain products of the FP64 arithmetic: every operation rounded as written,
-// so that a result has the same bits in every kernel, on the FP64 pipe (MulFp64)
-// or on the integer pipes (MulInt), which are otherwise idle.  mul0 is for operands that can be
-// tiny or zero (a product below the normal range is zero in both).
-struct MulFp64 {
-  static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
-  static __device__ __forceinline__ double mul0(double a, double b) { return mul_fp64_0(a, b); }
-  static __device__ __forceinline__ double half(double a) { return __dmul_rn(0.5, a); }
-};
-struct MulInt {
-  static __device__ __forceinline__ double mul(double a, double b) { return mul_int(a, b); }
-  static __device__ __forceinline__ double mul0(double a, double b) { return mul_int0(a, b); }
-  static __device__ __forceinline__ double half(double a) {  // exponent - 1
-    return __hiloint2double(__double2hiint(a) - (1 << 20), __double2loint(a));
-  }
-};
 
 // ---------------------------------------------------------------------------
 // HLLC flux across a face from the two sides' density r, normal velocity u,
@@ -497,14 +593,6 @@ __device__ __forceinline__ void hllc_axis(int D, const float (&qL)[5], const flo
   F[2] = x || z ? mf * qk[2] : fn;
   F[3] = z ? fn : mf * qk[3];
   F[4] = (eo + po) * uo;
-}
-
-// p <- max(p, r smallp), r > 0.  FP64: when p's exponent lies two above that
-// of r smallp the floor cannot act, and its product is not formed
-__device__ __forceinline__ float floor_p(float p, float r, float smallp) { return vmax(p, r * smallp); }
-__device__ __forceinline__ double floor_p(double p, double r, double smallp) {
-  if (__double2hiint(p) <= __double2hiint(r) + (__double2hiint(smallp) - (1021 << 20))) p = vmax(p, r * smallp);
-  return p;
 }
 
 // face states W* +- dW/2 of the two cells of a face (with the floors) and
