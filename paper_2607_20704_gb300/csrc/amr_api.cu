@@ -921,6 +921,7 @@ static CflArgs cfl_args(amr_mesh *h) {
   a.mgamma_t = h->mgamma_t;
   a.msmallr_t = h->msmallr_t;
   a.msmallp_t = h->msmallp_t;
+  a.mflag32 = h->mflag32;
   a.mlmin = h->mlmin;
   a.nmembers = h->M;
   a.smax = h->smax;
@@ -937,12 +938,13 @@ static CflArgs cfl_args(amr_mesh *h) {
 static void cfl_device(amr_mesh *h, int consume) {
   CflArgs a = cfl_args(h);
   a.consume = consume;
-  const unsigned grid = unsigned(std::min(a.ntiles, 4 * h->sm_count));
+  // the GPU filled twice over (2048 threads per SM): the pass waits on its loads
+  const unsigned grid = unsigned(std::min(a.ntiles, 4096 / h->tile_size * h->sm_count));
   if (grid) {
     if (h->p.precision == 4)
-      launch(h, K_CFL, k_cfl<float>, dim3(grid), dim3(unsigned(h->tile_size)), a, (const float *)h->U);
+      launch(h, K_CFL, k_cfl_fp32, dim3(grid), dim3(unsigned(h->tile_size)), a, (const float *)h->U);
     else
-      launch(h, K_CFL, k_cfl<double>, dim3(grid), dim3(unsigned(h->tile_size)), a, (const double *)h->U);
+      launch(h, K_CFL, k_cfl_fp64, dim3(grid), dim3(unsigned(h->tile_size)), a, (const double *)h->U);
   }
   launch(h, K_DT, k_dt, dim3(nblocks(h->M, 128)), dim3(128), a);
 }

@@ -89,6 +89,7 @@ struct CflArgs {
   const uint32_t *son;
   const double *mgamma, *msmallr, *msmallp, *mcfl;
   const void *mgamma_t, *msmallr_t, *msmallp_t;  // the same in the state's type
+  const float *mflag32;  // [3 members] gamma - 1, smallr, smallp rounded to FP32
   const int *mlmin;
   int nmembers;
   unsigned long long *smax;  // [16 * members] bit patterns of per-level maxima

@@ -113,6 +113,24 @@ __device__ __forceinline__ float rsqrt_nr(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double sound_speed(double c2) { return c2 > 0.0 ? c2 * rsqrt_nr(c2) : sqrt(c2); }
 __device__ __forceinline__ float sound_speed(float c2) { return sqrtf(c2); }
 
+// FP32 image of a state component: exact for an FP32 state; for FP64 the
+// bits are truncated on the integer pipes (relative error below 2^-23, no
+// conversion instruction: those run on the FP64 pipe), magnitudes below
+// 2^-126 give 0 and above 2^128 infinity
+template <class T>
+__device__ __forceinline__ float to_f32(T x) {
+  return float(x);
+}
+template <>
+__device__ __forceinline__ float to_f32<double>(double x) {
+  const uint64_t b = uint64_t(__double_as_longlong(x));
+  const uint32_t sign = uint32_t(b >> 32) & 0x80000000u;
+  const int e = int((b >> 52) & 0x7FF);
+  if (e < 1023 - 126) return __uint_as_float(sign);
+  if (e > 1023 + 127) return __uint_as_float(sign | 0x7F800000u);
+  return __uint_as_float(sign | (uint32_t(e - 896) << 23) | uint32_t((b >> 29) & 0x7FFFFFu));
+}
+
 // ---------------------------------------------------------------------------
 // segment context: what a thread needs to know about its (member, level)
 // ---------------------------------------------------------------------------
@@ -834,41 +852,43 @@ __device__ __forceinline__ void cfl_flush(const CflArgs &a, double s, int seg, d
   __syncthreads();
 }
 
-// Each block keeps a running maximum per thread while its tiles stay in one
-// segment and reduces it (one atomicMax) when the segment changes.
-// The running maximum is kept in the state's type (float to double is exact
-// and monotonic, so converting once per flush gives the same maximum) and
-// the parameters are read in that type: no conversions per cell, which would
-// run on the FP64 pipe.
+// sum_d (|u_d| + c) of a cell in the state's precision
 template <class T>
-__global__ void k_cfl(CflArgs a, const T *U) {
+__device__ __forceinline__ T cell_speed(T g, T smallr, T smallp, T u0, T u1, T u2, T u3, T u4) {
+  const T r = vmax(u0, smallr);
+  const T ir = rcp(r);
+  const T vx = u1 * ir, vy = u2 * ir, vz = u3 * ir;
+  const T ek = T(0.5) * r * ((vx * vx + vy * vy) + vz * vz);
+  const T p = vmax((g - T(1)) * (u4 - ek), r * smallp);
+  const T cs = sound_speed(g * p * ir);
+  return ((fabs(vx) + cs) + (fabs(vy) + cs)) + (fabs(vz) + cs);
+}
+
+// FP32: each block keeps a running maximum per thread while its tiles stay in
+// one segment and reduces it (one atomicMax) when the segment changes.
+// The running maximum is kept in FP32 (float to double is exact and monotonic,
+// so converting once per flush gives the same maximum) and the parameters are
+// read in that type: no conversions per cell, which would run on the FP64 pipe.
+__global__ void k_cfl_fp32(CflArgs a, const float *U) {
   __shared__ double wmax[32];
-  T s = T(0);
+  float s = 0.0f;
   int cur = -1;
-  const T *mgamma = static_cast<const T *>(a.mgamma_t), *msmallr = static_cast<const T *>(a.msmallr_t),
-          *msmallp = static_cast<const T *>(a.msmallp_t);
+  const float *mgamma = static_cast<const float *>(a.mgamma_t), *msmallr = static_cast<const float *>(a.msmallr_t),
+              *msmallp = static_cast<const float *>(a.msmallp_t);
   for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
     const Tile td = tile_at(a.tpre, a.tseg0, a.tnseg, a.tstep, ti);
     if (td.seg != cur) {
-      if (cur >= 0) cfl_flush<T>(a, double(s), cur, wmax);
-      s = T(0);
+      if (cur >= 0) cfl_flush<float>(a, double(s), cur, wmax);
+      s = 0.0f;
       cur = td.seg;
     }
     const Seg sg = a.segs[td.seg];
     const int t = td.start + threadIdx.x;
     if (t < 8 * sg.nl && a.mrem[sg.member] != 0 &&
         !((__ldg(a.son + sg.lo + (t >> 3)) >> (t & 7)) & 1u)) {
-      const T g = mgamma[sg.member], smallr = msmallr[sg.member], smallp = msmallp[sg.member];
       const int64_t gi = 8 * int64_t(sg.lo) + t;
-      const T u0 = U[gi], u1 = U[a.S + gi], u2 = U[2 * a.S + gi], u3 = U[3 * a.S + gi],
-              u4 = U[4 * a.S + gi];
-      const T r = vmax(u0, smallr);
-      const T ir = rcp(r);
-      const T vx = u1 * ir, vy = u2 * ir, vz = u3 * ir;
-      const T ek = T(0.5) * r * ((vx * vx + vy * vy) + vz * vz);
-      const T p = vmax((g - T(1)) * (u4 - ek), r * smallp);
-      const T cs = sound_speed(g * p * ir);
-      const T st = ((fabs(vx) + cs) + (fabs(vy) + cs)) + (fabs(vz) + cs);
+      const float u0 = U[gi], u1 = U[a.S + gi], u2 = U[2 * a.S + gi], u3 = U[3 * a.S + gi], u4 = U[4 * a.S + gi];
+      const float st = cell_speed(mgamma[sg.member], msmallr[sg.member], msmallp[sg.member], u0, u1, u2, u3, u4);
       if (!finite_bits(st) || !(finite_bits(u0) && finite_bits(u1) && finite_bits(u2) &&
                                 finite_bits(u3) && finite_bits(u4))) {
         atomicOr(a.err, kErrNaN);
@@ -878,7 +898,78 @@ __global__ void k_cfl(CflArgs a, const T *U) {
       }
     }
   }
-  if (cur >= 0) cfl_flush<T>(a, double(s), cur, wmax);
+  if (cur >= 0) cfl_flush<float>(a, double(s), cur, wmax);
+}
+
+// FP64: the maximum needs the FP64 speed of few cells.  Each cell's speed is
+// bounded from above in FP32; a warp forms the FP64 speeds (31 operations on
+// the FP64 pipe, which bounded this pass) only when one of its bounds reaches
+// the largest speed found so far, and publishes what it finds at once.  The
+// maximum is over the same FP64 values as before: a cell passed over lies
+// strictly below one of them.
+//
+// The bound: the FP32 images of the state are truncated (relative error below
+// 2^-23), the parameters, quotients, squares and sums err by a few 2^-23 each:
+// |u_d| by less than 2^-20 of itself, ek by less than 2^-19, so E - ek lies
+// within 2^-18 (|E| + ek) of its FP32 value; c = sqrt(gamma p / rho) by less
+// than 2^-18 of itself and sqrt(gamma smallp) for the floor.  2^-16 over the
+// sum covers them and the approximate reciprocal, and 2^-60 a momentum that
+// vanishes in FP32.  A cell whose density, energy, kinetic energy or gamma lies
+// outside the powers of two named below (no value there over- or underflows),
+// or that is not finite, always takes the FP64 test: an infinite or NaN
+// momentum makes its kinetic energy so.
+__global__ void __launch_bounds__(512) k_cfl_fp64(CflArgs a, const double *U) {
+  const double *mgamma = a.mgamma, *msmallr = a.msmallr, *msmallp = a.msmallp;
+  for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tpre, a.tseg0, a.tnseg, a.tstep, ti);
+    const Seg sg = a.segs[td.seg];
+    const int t = td.start + threadIdx.x;
+    unsigned long long *out = a.smax + 16 * sg.member + sg.level;
+    bool test = false;
+    double u0 = 0.0, u1 = 0.0, u2 = 0.0, u3 = 0.0, u4 = 0.0;
+    if (t < 8 * sg.nl && a.mrem[sg.member] != 0 &&
+        !((__ldg(a.son + sg.lo + (t >> 3)) >> (t & 7)) & 1u)) {
+      const unsigned long long seen = __ldcg(out);
+      const int64_t gi = 8 * int64_t(sg.lo) + t;
+      u0 = U[gi];
+      u1 = U[a.S + gi];
+      u2 = U[2 * a.S + gi];
+      u3 = U[3 * a.S + gi];
+      u4 = U[4 * a.S + gi];
+      const float gm1 = a.mflag32[3 * sg.member], smallr = a.mflag32[3 * sg.member + 1],
+                  smallp = a.mflag32[3 * sg.member + 2];
+      const float g = gm1 + 1.0f;
+      const float r = fmaxf(to_f32(u0), smallr), ir = rcp(r);
+      const float vx = fabsf(to_f32(u1)) * ir, vy = fabsf(to_f32(u2)) * ir, vz = fabsf(to_f32(u3)) * ir;
+      const float e4 = to_f32(u4), ek = 0.5f * r * ((vx * vx + vy * vy) + vz * vz);
+      const float p = gm1 * ((e4 - ek) + 0x1p-18f * (fabsf(e4) + ek));
+      const float c = sqrtf(g * fmaxf(p, 0.0f) * ir) + sqrtf(g * smallp);
+      const float bound = (1.0f + 0x1p-16f) * ((vx + vy) + (vz + 3.0f * c)) + 0x1p-60f;
+      const bool ok = r >= 0x1p-60f && r <= 0x1p60f && e4 >= 0x1p-60f && e4 <= 0x1p60f && ek <= 0x1p60f &&
+                      gm1 >= 0x1p-20f && gm1 <= 0x1p20f && finite_bits(u0);
+      test = !ok || !(bound < to_f32(__longlong_as_double((long long)seen)));
+    }
+    if (!__any_sync(0xFFFFFFFFu, test)) continue;
+    double s = 0.0;
+    if (test) {
+      s = cell_speed(__ldg(mgamma + sg.member), __ldg(msmallr + sg.member), __ldg(msmallp + sg.member), u0, u1, u2,
+                     u3, u4);
+      if (!finite_bits(s) || !(finite_bits(u0) && finite_bits(u1) && finite_bits(u2) && finite_bits(u3) &&
+                               finite_bits(u4))) {
+        atomicOr(a.err, kErrNaN);
+        atomicOr(a.merr + sg.member, kErrNaN);
+        s = 0.0;
+      }
+    }
+    // the warp's maximum: non-negative doubles order like their bits
+    long long b = __double_as_longlong(s);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const long long o = __shfl_xor_sync(0xFFFFFFFFu, b, off);
+      b = o > b ? o : b;
+    }
+    if ((threadIdx.x & 31) == 0 && b > 0) atomicMax(out, (unsigned long long)b);
+  }
 }
 
 __global__ void k_dt(CflArgs a) {

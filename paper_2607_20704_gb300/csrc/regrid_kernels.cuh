@@ -100,24 +100,6 @@ __device__ __forceinline__ void load_cell(const T *U, int64_t S, int64_t g, doub
 // about ten times that), and 2^-21 p for the floor rho smallp (max is
 // 1-Lipschitz).  A cell whose values leave [2^-60, 2^60] gets the bound
 // +inf: its tests always run in FP64.
-// FP32 image of a state component: exact for an FP32 state; for FP64 the
-// bits are truncated on the integer pipes (relative error below 2^-23, no
-// conversion instruction: those run on the FP64 pipe), magnitudes below
-// 2^-126 give 0 and above 2^128 infinity
-template <class T>
-__device__ __forceinline__ float to_f32(T x) {
-  return float(x);
-}
-template <>
-__device__ __forceinline__ float to_f32<double>(double x) {
-  const uint64_t b = uint64_t(__double_as_longlong(x));
-  const uint32_t sign = uint32_t(b >> 32) & 0x80000000u;
-  const int e = int((b >> 52) & 0x7FF);
-  if (e < 1023 - 126) return __uint_as_float(sign);
-  if (e > 1023 + 127) return __uint_as_float(sign | 0x7F800000u);
-  return __uint_as_float(sign | (uint32_t(e - 896) << 23) | uint32_t((b >> 29) & 0x7FFFFFu));
-}
-
 __device__ __forceinline__ bool in_range32(float x) { return x >= 0x1p-60f && x <= 0x1p60f; }
 
 template <class T>
