@@ -136,7 +136,8 @@ struct HostPin {
 
 // level-step launch domains of a segment
 enum Dom {
-  DOM_CELLS = 0, DOM_REAL = 1, DOM_GHOST5 = 2, DOM_POST = 3, DOM_BLOCKS = 4, DOM_COMMIT = 5, DOM_COUNT = 6
+  DOM_CELLS = 0, DOM_REAL = 1, DOM_GHOST5 = 2, DOM_UPDATE = 3, DOM_BLOCKS = 4, DOM_COMMIT = 5, DOM_RESTRICT = 6,
+  DOM_REFLUX = 7, DOM_COUNT = 8
 };
 
 // a list of segments and, per domain, its tiles: the offset of its tile
@@ -144,7 +145,7 @@ enum Dom {
 // number of tiles
 struct SegList {
   int seg0 = 0, nseg = 0;
-  int tpre0[DOM_COUNT] = {0, 0, 0, 0, 0, 0}, ntile[DOM_COUNT] = {0, 0, 0, 0, 0, 0};
+  int tpre0[DOM_COUNT] = {}, ntile[DOM_COUNT] = {};
   int ls = 0;  // scratch cells used
 };
 
@@ -631,8 +632,9 @@ static int dom_size(const Seg &s, int dom) {
     case DOM_GHOST5: return 5 * s.ncl;
     case DOM_BLOCKS: return s.nblk;
     case DOM_COMMIT: return ((s.flags & kSegReflux) ? 5 * s.ncl : 0) + 5 * s.nl;
-    default:
-      return ((s.flags & kSegReflux) ? 5 * s.ncl : 0) + ((s.flags & kSegRestrict) ? 5 * s.nl : 0);
+    case DOM_UPDATE: return 8 * s.nl + ((s.flags & kSegReflux) ? 5 * s.ncl : 0);
+    case DOM_REFLUX: return (s.flags & kSegReflux) ? 5 * s.ncl : 0;
+    default: return (s.flags & kSegRestrict) ? 5 * s.nl : 0;
   }
 }
 
@@ -738,14 +740,17 @@ static void build_lists(amr_mesh *h) {
 // ---------------------------------------------------------------------------
 // level-step launches
 // ---------------------------------------------------------------------------
-// the tiles of domain `dom` of list L in the launch arguments
-template <class A>
-static void set_tiles(amr_mesh *h, A &a, const SegList &L, int dom) {
-  a.tpre = h->tpre + L.tpre0[dom];
-  a.tseg0 = L.seg0;
-  a.tnseg = L.nseg;
-  a.tstep = dom == DOM_BLOCKS ? 1 : h->tile_size;
-  a.ntiles = L.ntile[dom];
+// the tiles of domain `dom` of list L
+static TileList tile_list(amr_mesh *h, const SegList &L, int dom) {
+  TileList t{};
+  t.segs = h->segs;
+  t.tpre = h->tpre + L.tpre0[dom];
+  t.seg0 = L.seg0;
+  t.nseg = L.nseg;
+  t.step = dom == DOM_BLOCKS ? 1 : h->tile_size;
+  t.ntiles = L.ntile[dom];
+  if (L.nseg == 1) t.one = h->segs_h[size_t(L.seg0)];
+  return t;
 }
 
 template <class T>
@@ -770,7 +775,6 @@ static StepArgs<T> step_args(amr_mesh *h, bool device_dt, double dt) {
   a.Q = static_cast<T *>(h->Q);
   a.F = static_cast<T *>(h->F);
   a.C = static_cast<T *>(h->C);
-  a.segs = h->segs;
   a.mgamma = static_cast<const T *>(h->mgamma_t);
   a.migm1 = static_cast<const T *>(h->migm1_t);
   a.msmallr = static_cast<const T *>(h->msmallr_t);
@@ -784,35 +788,37 @@ static StepArgs<T> step_args(amr_mesh *h, bool device_dt, double dt) {
   return a;
 }
 
-// persistent grid: enough blocks to fill the GPU once, never more than tiles
+// persistent grid: enough blocks to fill the GPU once, never more than tiles;
+// smem: bytes of dynamic shared memory per thread
 template <class T>
 static void run_list(amr_mesh *h, int kid, void (*kern)(StepArgs<T>), StepArgs<T> a,
-                     const SegList &L, int dom) {
+                     const SegList &L, int dom, size_t smem = 0) {
   if (L.ntile[dom] == 0) return;
-  set_tiles(h, a, L, dom);
-  int grid = a.ntiles;
+  a.tiles = tile_list(h, L, dom);
+  int grid = a.tiles.ntiles;
   if (h->persistent) {
     int per_sm = 0;
     for (auto &o : h->occ)
       if (o.first == (const void *)kern) per_sm = o.second;
     if (per_sm == 0) {
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, h->tile_size, 0) != cudaSuccess ||
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, h->tile_size, smem * h->tile_size) !=
+              cudaSuccess ||
           per_sm < 1) {
         cudaGetLastError();
         per_sm = 1;
       }
       h->occ.push_back({(const void *)kern, per_sm});
     }
-    grid = std::min(a.ntiles, per_sm * h->sm_count);
+    grid = std::min(a.tiles.ntiles, per_sm * h->sm_count);
   }
-  launch(h, kid, kern, dim3(unsigned(grid)), dim3(unsigned(h->tile_size)), a);
+  launch_smem(h, kid, kern, dim3(unsigned(grid)), dim3(unsigned(h->tile_size)), smem * h->tile_size, a);
 }
 
 // the fused kernel over the blocks of a list (dynamic shared memory)
 template <class T, int NS>
 static void run_rock_ns(amr_mesh *h, StepArgs<T> a, const SegList &L) {
   if (L.ntile[DOM_BLOCKS] == 0) return;
-  set_tiles(h, a, L, DOM_BLOCKS);
+  a.tiles = tile_list(h, L, DOM_BLOCKS);
   constexpr size_t smem = Rock<NS>::template smem<T>();
   auto kern = k_rock<T, NS>;
   int per_sm = 0;
@@ -827,7 +833,7 @@ static void run_rock_ns(amr_mesh *h, StepArgs<T> a, const SegList &L) {
     }
     h->occ.push_back({(const void *)kern, per_sm});
   }
-  const int grid = h->persistent ? std::min(a.ntiles, per_sm * h->sm_count) : a.ntiles;
+  const int grid = h->persistent ? std::min(a.tiles.ntiles, per_sm * h->sm_count) : a.tiles.ntiles;
   launch_smem(h, K_ROCK, kern, dim3(unsigned(grid)), dim3(unsigned(Rock<NS>::THREADS)), smem, a,
               (const int32_t *)h->blk);
 }
@@ -835,7 +841,7 @@ static void run_rock_ns(amr_mesh *h, StepArgs<T> a, const SegList &L) {
 template <class T, int NS>
 static void run_sweep_ns(amr_mesh *h, StepArgs<T> a, const SegList &L) {
   if (L.ntile[DOM_BLOCKS] == 0) return;
-  set_tiles(h, a, L, DOM_BLOCKS);
+  a.tiles = tile_list(h, L, DOM_BLOCKS);
   constexpr size_t smem = Sweep<NS>::template smem<T>();
   auto kern = k_sweep<T, NS>;
   int per_sm = 0;
@@ -850,16 +856,30 @@ static void run_sweep_ns(amr_mesh *h, StepArgs<T> a, const SegList &L) {
     }
     h->occ.push_back({(const void *)kern, per_sm});
   }
-  const int grid = h->persistent ? std::min(a.ntiles, per_sm * h->sm_count) : a.ntiles;
+  const int grid = h->persistent ? std::min(a.tiles.ntiles, per_sm * h->sm_count) : a.tiles.ntiles;
   launch_smem(h, K_SWEEP, kern, dim3(unsigned(grid)), dim3(unsigned(Sweep<NS>::THREADS)), smem, a,
               (const int32_t *)h->blk);
 }
 
+// the ghost octs of a list, and the reflux sums of another
 template <class T>
-static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double dt) {
+static void run_prolong(amr_mesh *h, StepArgs<T> a, const SegList &L, const SegList *pend) {
+  a.tiles = tile_list(h, L, DOM_GHOST5);
+  TileList p{};
+  if (pend) p = tile_list(h, *pend, DOM_REFLUX);
+  const int grid = std::max(a.tiles.ntiles, p.ntiles);
+  if (grid == 0) return;
+  launch(h, K_PROLONG, k_prolong<T>, dim3(unsigned(grid)), dim3(unsigned(h->tile_size)), a, p);
+}
+
+template <class T>
+static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double dt, const SegList **pend) {
   if (L.nseg == 0) return;
   StepArgs<T> a = step_args<T>(h, device_dt, dt);
-  run_list(h, K_PROLONG, k_prolong<T>, a, L, DOM_GHOST5);
+  if (h->nsub > 0 || sizeof(T) == 4) {
+    run_prolong<T>(h, a, L, *pend);
+    *pend = nullptr;
+  }
   if (h->nsub > 0) {
     // the paper's fused kernels (cube staging or planar sweep): one block of
     // nsub^3 octs per CTA, then the new leaf states from the scratch into U
@@ -884,34 +904,40 @@ static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double d
     // FP32: primitives recomputed inside the predictor; each leaf cell solves
     // its six faces and updates itself
     run_list(h, K_PREDICT, k_predict_u<T>, a, L, DOM_CELLS);
-    run_list(h, K_FLUX, k_flux_update<T>, a, L, DOM_REAL);
+    run_list(h, K_FLUX, k_flux_update, a, L, DOM_REAL, 20);
+    if (L.ntile[DOM_REFLUX]) *pend = &L;
   } else {
     // FP64: every predictor and every face solve exactly once
-    run_list(h, K_PRIM, k_prim<T>, a, L, DOM_CELLS);
+    run_list(h, K_PRIM, k_ghost_prim, a, L, DOM_CELLS, 16);
     run_list(h, K_PREDICT, k_predict, a, L, DOM_CELLS);
     run_list(h, K_FLUX, k_flux<T>, a, L, DOM_CELLS);
-    run_list(h, K_UPDATE, k_update<T>, a, L, DOM_REAL);
+    run_list(h, K_UPDATE, k_update, a, L, DOM_UPDATE, 40);
   }
-  run_list(h, K_RESTRICT, k_reflux_restrict<T>, a, L, DOM_POST);
 }
 
-static void step_segments(amr_mesh *h, const SegList &L, bool device_dt, double dt) {
+// One level step of a list.  *pend: a list whose reflux sums are still to be
+// formed, taken over by this step; the step may leave its own (see flush_reflux).
+static void step_segments(amr_mesh *h, const SegList &L, bool device_dt, double dt, const SegList **pend) {
   if (h->p.precision == 4)
-    run_segments<float>(h, L, device_dt, dt);
+    run_segments<float>(h, L, device_dt, dt, pend);
   else
-    run_segments<double>(h, L, device_dt, dt);
+    run_segments<double>(h, L, device_dt, dt, pend);
+}
+
+// the reflux sums that the last level step left (FP32)
+static void flush_reflux(amr_mesh *h, bool device_dt, const SegList *pend) {
+  if (pend) run_list(h, K_REFLUX, k_reflux<float>, step_args<float>(h, device_dt, 0.0), *pend, DOM_REFLUX);
 }
 
 template <class T>
 static void restrict_segments(amr_mesh *h, const SegList &L) {
   if (L.nseg == 0) return;
-  run_list(h, K_RESTRICT, k_reflux_restrict<T>, step_args<T>(h, false, 0.0), L, DOM_POST);
+  run_list(h, K_RESTRICT, k_restrict<T>, step_args<T>(h, false, 0.0), L, DOM_RESTRICT);
 }
 
 static CflArgs cfl_args(amr_mesh *h) {
   CflArgs a{};
-  a.segs = h->segs;
-  set_tiles(h, a, h->cfl_list, DOM_REAL);
+  a.tiles = tile_list(h, h->cfl_list, DOM_REAL);
   a.S = h->S;
   a.son = h->son;
   a.mgamma = h->mgamma_d;
@@ -939,7 +965,7 @@ static void cfl_device(amr_mesh *h, int consume) {
   CflArgs a = cfl_args(h);
   a.consume = consume;
   // the GPU filled twice over (2048 threads per SM): the pass waits on its loads
-  const unsigned grid = unsigned(std::min(a.ntiles, 4096 / h->tile_size * h->sm_count));
+  const unsigned grid = unsigned(std::min(a.tiles.ntiles, 4096 / h->tile_size * h->sm_count));
   if (grid) {
     if (h->p.precision == 4)
       launch(h, K_CFL, k_cfl_fp32, dim3(grid), dim3(unsigned(h->tile_size)), a, (const float *)h->U);
@@ -1658,7 +1684,9 @@ extern "C" amr_status amr_step_level(amr_handle h, int level, double dt) {
   if (level < 1 || level > h->lmax_all)
     return fail(AMR_EINVAL, "amr_step_level: level %d outside [1, %d]", level, h->lmax_all);
   if (!(dt > 0.0)) return fail(AMR_EINVAL, "amr_step_level: dt must be > 0");
-  step_segments(h, h->level_list[level], false, dt);
+  const SegList *pend = nullptr;
+  step_segments(h, h->level_list[level], false, dt, &pend);
+  flush_reflux(h, false, pend);
   if (h->launch_err != cudaSuccess) return check_device(h, "amr_step_level");
   return AMR_OK;
 }
@@ -1666,7 +1694,9 @@ extern "C" amr_status amr_step_level(amr_handle h, int level, double dt) {
 static void coarse_step(amr_mesh *h) {
   if (h->p.reindex_every_step) reindex(h);
   cfl_device(h, 1);
-  for (auto &L : h->phases) step_segments(h, L, true, 0.0);
+  const SegList *pend = nullptr;
+  for (auto &L : h->phases) step_segments(h, L, true, 0.0, &pend);
+  flush_reflux(h, true, pend);
 }
 
 static void coarse_step(amr_mesh *h);
@@ -1983,9 +2013,9 @@ extern "C" amr_status amr_fill_ghosts(amr_handle h, int level) {
   if (level < 1 || level > kMaxLev) return fail(AMR_EINVAL, "amr_fill_ghosts: bad level");
   const SegList &L = h->level_list[level];
   if (h->p.precision == 4)
-    run_list(h, K_PROLONG, k_prolong<float>, step_args<float>(h, false, 0.0), L, DOM_GHOST5);
+    run_prolong<float>(h, step_args<float>(h, false, 0.0), L, nullptr);
   else
-    run_list(h, K_PROLONG, k_prolong<double>, step_args<double>(h, false, 0.0), L, DOM_GHOST5);
+    run_prolong<double>(h, step_args<double>(h, false, 0.0), L, nullptr);
   return AMR_OK;
 }
 

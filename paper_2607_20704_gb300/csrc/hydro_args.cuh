@@ -23,25 +23,40 @@ enum : int { kSegReflux = 1, kSegRestrict = 2 };
 // A launch covers a flattened list of tiles; tile (seg, start) is the block
 // of domain items [start, start + step) of segment seg.  A list stores only
 // its segments' cumulative tile counts (tpre[q] = first tile of its q-th
-// segment, tpre[nseg] = all tiles); a kernel finds the segment of tile ti by
-// binary search.
+// segment, tpre[nseg] = all tiles); a kernel finds the segment of tile ti as
+// the last one whose first tile is <= ti (segments without tiles share their
+// successor's first tile and are passed over).
 struct Tile {
   int seg, start;
 };
 
-// the last segment of the list whose first tile is <= ti (segments without
-// tiles share their successor's first tile and are passed over)
-__device__ __forceinline__ Tile tile_at(const int *__restrict__ tpre, int seg0, int nseg, int step, int ti) {
-  int lo = 0, hi = nseg - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(tpre + mid) <= ti)
-      lo = mid;
-    else
-      hi = mid - 1;
+// a launch's list: its first segment and their number, items per tile, tiles;
+// a list of one segment (a mesh on its own) carries it as an argument, so that
+// a small level's kernels do not wait for the list's loads before their own
+struct TileList {
+  const Seg *segs;
+  const int *tpre;
+  int seg0, nseg, step, ntiles;
+  Seg one;
+};
+
+// called by whole warps with the same ti: counts 32 segments per round (the
+// loads of a round are independent; a bisection would chain them)
+__device__ __forceinline__ Tile tile_at(const TileList &l, int ti) {
+  if (l.nseg == 1) return Tile{l.seg0, ti * l.step};
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = l.nseg;  // the segment lies in [lo, lo + n)
+  while (n > 1) {
+    const int stride = (n + 31) >> 5;
+    const int q = lane * stride;
+    const bool le = q < n && __ldg(l.tpre + lo + q) <= ti;
+    const int k = __popc(__ballot_sync(0xFFFFFFFFu, le)) - 1;
+    lo += k * stride;
+    n = n - k * stride < stride ? n - k * stride : stride;
   }
-  return Tile{seg0 + lo, (ti - __ldg(tpre + lo)) * step};
+  return Tile{l.seg0 + lo, (ti - __ldg(l.tpre + lo)) * l.step};
 }
+__device__ __forceinline__ Seg seg_at(const TileList &l, int seg) { return l.nseg == 1 ? l.one : l.segs[seg]; }
 
 // Everything a level-step launch needs, passed by value.  Oct counts and cell
 // indices fit in 32 bits (at most 2^26 real octs, and 8 (real + ghost octs)
@@ -64,9 +79,7 @@ struct StepArgs {
   const uint64_t *key;    // [N] internal keys
   const int32_t *csrc;    // [7][NC] prolongation sources (global cell indices)
   T *W, *Q, *F, *C;       // scratch W[5][LS], Q[20][LS], F[15][LS]; slots C[5][CS]
-  const Seg *segs;
-  const int *tpre;                  // the list's tile prefix (see Tile)
-  int tseg0, tnseg, tstep, ntiles;  // first segment, segments, items per tile, tiles
+  TileList tiles;
   // per member: gamma, {1/(gamma-1), gamma-1}, floors
   const T *mgamma, *migm1, *msmallr, *msmallp;
   // dt/dx: from the device time step of each member's coarse step
@@ -82,9 +95,7 @@ struct StepArgs {
 };
 
 struct CflArgs {
-  const Seg *segs;
-  const int *tpre;
-  int tseg0, tnseg, tstep, ntiles;
+  TileList tiles;
   int64_t S;
   const uint32_t *son;
   const double *mgamma, *msmallr, *msmallp, *mcfl;

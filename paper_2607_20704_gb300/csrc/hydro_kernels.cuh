@@ -3,15 +3,17 @@
 // ghost cells per side; Sec. 2.3 ghost octs; Table 1 stages godunov /
 // set uold / upload), as non-redundant per-cell passes:
 //
-//   k_prolong   ghost octs of the level from their father cell (minmod)
-//   k_prim      primitive variables of every real and ghost cell
-//   k_predict   limited slopes and the Hancock half-step, once per cell
-//   k_flux      one HLLC flux per face (owned by the cell on its minus side)
-//   k_update    conservative update of leaf cells + pending reflux
-//   k_reflux_restrict  fixed-order sum of coarse-fine fluxes for the coarse
-//               cells, and father cell = mean of its 8 children
+//   k_ghost_prim  ghost octs of the level from their father cell (minmod) and
+//                 primitive variables of every real and ghost cell
+//   k_predict     limited slopes and the Hancock half-step, once per cell
+//   k_flux        one HLLC flux per face (owned by the cell on its minus side)
+//   k_update      conservative update of leaf cells + pending reflux; father
+//                 cell = mean of its 8 children; fixed-order sum of
+//                 coarse-fine fluxes for the coarse cells
 //
-// (FP32 fuses k_prim into k_predict_u and k_flux with k_update.)
+// FP32 takes three: k_prolong (ghost octs, and the previous level step's
+// fixed-order sums of coarse-fine fluxes), k_predict_u (primitives formed from U
+// as they are needed) and k_flux_update (flux, update, father cells).
 //
 // The paper's kernels gather a 6x6x6 stencil per oct and recompute the
 // slopes and predictor of its ghost ring (8x work per cell at nsubgrid=1).
@@ -149,8 +151,7 @@ __device__ __forceinline__ float seg_dtdx(const StepArgs<float> &a, const Seg &s
 }
 
 template <class T>
-__device__ __forceinline__ SegCtx<T> seg_ctx(const StepArgs<T> &a, int seg) {
-  const Seg s = a.segs[seg];
+__device__ __forceinline__ SegCtx<T> seg_ctx(const StepArgs<T> &a, const Seg &s) {
   SegCtx<T> c;
   c.lo = s.lo;
   c.nl = s.nl;
@@ -171,10 +172,11 @@ __device__ __forceinline__ SegCtx<T> seg_ctx(const StepArgs<T> &a, int seg) {
 // the tile that lies inside the segment's domain of `size(ctx)` items
 template <class T, class Size, class Body>
 __device__ __forceinline__ void tile_loop(const StepArgs<T> &a, Size size, Body body) {
-  for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tpre, a.tseg0, a.tnseg, a.tstep, ti);
-    if (a.mact && !__ldg(a.mact + a.segs[td.seg].member)) continue;  // finished member
-    const SegCtx<T> sc = seg_ctx(a, td.seg);
+  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tiles, ti);
+    const Seg sg = seg_at(a.tiles, td.seg);
+    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
+    const SegCtx<T> sc = seg_ctx(a, sg);
 #ifdef AMR_CHECKED
     // the segment's local cells must fit the scratch arrays
     if (sc.base < 0 || sc.base + 8 * (sc.nl + sc.ncl) > a.LS) {
@@ -218,12 +220,44 @@ __device__ __forceinline__ bool cell_is_split(const StepArgs<T> &a, const SegCtx
   return (__ldg(a.son + s.lo + q) >> (t & 7)) & 1u;
 }
 
+// R(X) += sum of the 24 slots of ghost oct g (X its father cell), in slot
+// order (direction -x,+x,-y,+y,-z,+z seen from X, then fine face)
+template <class T>
+__device__ __forceinline__ void reflux_sum(const StepArgs<T> &a, int v, int g) {
+  const T *cv = a.C + v * a.CS + 24 * int64_t(g);
+  T *Rv = a.Rc + v * int64_t(a.NC) + g;
+  T acc = *Rv;
+#pragma unroll
+  for (int k = 0; k < 24; ++k) acc += cv[k];
+  *Rv = acc;
+}
+
+// the reflux sums of a list's ghost octs; domain: 5 ncl (if kSegReflux)
+template <class T>
+__device__ __forceinline__ void reflux_tile(const StepArgs<T> &a, const TileList &l, int ti) {
+  const Tile td = tile_at(l, ti);
+  const Seg s = seg_at(l, td.seg);
+  if (a.mact && !__ldg(a.mact + s.member)) return;  // finished member
+  const int q = td.start + threadIdx.x;
+  if (!(s.flags & kSegReflux) || q >= 5 * s.ncl) return;
+  const int v = q / s.ncl;
+  reflux_sum(a, v, s.clo + (q - v * s.ncl));
+}
+template <class T>
+__global__ void k_reflux(StepArgs<T> a) {
+  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) reflux_tile(a, a.tiles, ti);
+}
+
 // ---------------------------------------------------------------------------
 // ghost octs: child = U_C + sum_d (+-1/4) minmod(U(C+e_d)-U(C), U(C)-U(C-e_d))
 // domain: 5 * ncl (variable, ghost oct)
 // ---------------------------------------------------------------------------
+// pend: a list whose fluxes were solved by the previous level step and whose
+// reflux sums are still to be formed (FP32: the slots are written by the last
+// kernel of a level step); they touch other data, so they ride along here
 template <class T>
-__global__ void k_prolong(StepArgs<T> a) {
+__global__ void k_prolong(StepArgs<T> a, TileList pend) {
+  for (int ti = blockIdx.x; ti < pend.ntiles; ti += gridDim.x) reflux_tile(a, pend, ti);
   tile_loop(a, [](const SegCtx<T> &s) { return 5 * s.ncl; }, [&](const SegCtx<T> &s, int q) {
     const int v = q / s.ncl;
     const int cs = s.clo + (q - v * s.ncl);
@@ -321,16 +355,71 @@ __device__ __forceinline__ void prim_at(const StepArgs<T> &a, const SegCtx<T> &s
   prim_of(s, a.U[g], a.U[a.S + g], a.U[2 * a.S + g], a.U[3 * a.S + g], a.U[4 * a.S + g], w);
 }
 
-template <class T>
-__global__ void k_prim(StepArgs<T> a) {
-  tile_loop(a, [](const SegCtx<T> &s) { return 8 * (s.nl + s.ncl); },
-            [&](const SegCtx<T> &s, int t) {
-              T w[5];
-              prim_at(a, s, t, w);
-              const int o = s.base + t;
+// FP64: ghost octs (as k_prolong) and the primitives of every real and ghost
+// cell in one pass; thread per cell, an oct in 8 neighbouring lanes.  A ghost
+// oct's 15 slopes (variable, axis) are formed once, two per lane, and shared by
+// its cells.
+__global__ void __launch_bounds__(512, 3) k_ghost_prim(StepArgs<double> a) {
+  extern __shared__ double slopes[];  // [5 d + v][oct of the block], 16 bytes per thread
+  const int nq = blockDim.x >> 3;
+  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tiles, ti);
+    const Seg sg = seg_at(a.tiles, td.seg);
+    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
+    const SegCtx<double> s = seg_ctx(a, sg);
+#ifdef AMR_CHECKED
+    if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
+      atomicOr(a.err, kErrIndex);
+      continue;
+    }
+#endif
+    const int t = td.start + threadIdx.x;
+    const int q = t >> 3, c = t & 7, qb = threadIdx.x >> 3;
+    const bool on = t < 8 * (s.nl + s.ncl), ghost = on && q >= s.nl;
+    const int cs = s.clo + (q - s.nl);
+    const int64_t g = 8 * int64_t(ext_of_local(a, s, q)) + c;
+    double u[5];
+    if (ghost) {
 #pragma unroll
-              for (int v = 0; v < 5; ++v) a.W[v * a.LS + o] = w[v];
-            });
+      for (int h = 0; h < 2; ++h) {
+        const int k = c + 8 * h;  // slope 5 d + v
+        if (k < 15) {
+          const int d = k / 5;
+          const double *Uv = a.U + (k - 5 * d) * a.S;
+          auto at = [&](int j) {
+            return Uv[checked(__ldg(a.csrc + j * int64_t(a.NC) + cs), 0, 8 * int64_t(a.NE), a.err)];
+          };
+          const double uc = at(0), um = at(1 + 2 * d), up = at(2 + 2 * d);
+          slopes[k * nq + qb] = minmod(up - uc, uc - um);
+        }
+      }
+      const int64_t f = checked(__ldg(a.csrc + cs), 0, 8 * int64_t(a.NE), a.err);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + f];
+    } else if (on) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + g];
+    }
+    if (__any_sync(0xFFFFFFFFu, ghost)) {
+      __syncwarp();
+      if (ghost) {
+        const double hx = (c & 1) ? 0.25 : -0.25, hy = (c & 2) ? 0.25 : -0.25, hz = (c & 4) ? 0.25 : -0.25;
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          u[v] = ((u[v] + hx * slopes[v * nq + qb]) + hy * slopes[(5 + v) * nq + qb]) + hz * slopes[(10 + v) * nq + qb];
+          a.U[v * a.S + g] = u[v];
+        }
+      }
+      __syncwarp();
+    }
+    if (on) {
+      double w[5];
+      prim_of(s, u[0], u[1], u[2], u[3], u[4], w);
+      const int o = s.base + t;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) a.W[v * a.LS + o] = w[v];
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -409,10 +498,11 @@ __device__ __forceinline__ double shfl_xor_f64(unsigned mask, double x, int lane
   return __hiloint2double(hi, lo);
 }
 __global__ void k_predict(StepArgs<double> a) {
-  for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tpre, a.tseg0, a.tnseg, a.tstep, ti);
-    if (a.mact && !__ldg(a.mact + a.segs[td.seg].member)) continue;  // finished member
-    const SegCtx<double> s = seg_ctx(a, td.seg);
+  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tiles, ti);
+    const Seg sg = seg_at(a.tiles, td.seg);
+    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
+    const SegCtx<double> s = seg_ctx(a, sg);
 #ifdef AMR_CHECKED
     if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
       atomicOr(a.err, kErrIndex);
@@ -697,13 +787,10 @@ __global__ void k_flux(StepArgs<T> a) {
             });
 }
 
-// U <- (U + dt/dx sum_d (F_d- - F_d+)) + R on leaf cells; R <- 0.  The new
-// state goes to `out` (stride `ostride`): U itself, or a buffer when other
-// blocks may still read the old state.
+// U <- (U + dt/dx sum_d (F_d- - F_d+)) + R on leaf cells; R <- 0
 template <class T>
-__device__ __forceinline__ void update_cell_to(const StepArgs<T> &a, const SegCtx<T> &s, int g,
-                                               const T (&dx)[5], const T (&dy)[5], const T (&dz)[5],
-                                               T *out, int64_t ostride) {
+__device__ __forceinline__ void new_state(const StepArgs<T> &a, const SegCtx<T> &s, int g, const T (&dx)[5],
+                                          const T (&dy)[5], const T (&dz)[5], T (&un)[5]) {
   const int rs = int(checked(__ldg(a.rslot + g), -1, a.NC, a.err, -1));
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
@@ -713,33 +800,95 @@ __device__ __forceinline__ void update_cell_to(const StepArgs<T> &a, const SegCt
       u = u + *Rv;
       *Rv = T(0);
     }
-    out[v * ostride] = u;
+    un[v] = u;
+  }
+}
+template <class T>
+__device__ __forceinline__ void update_cell(const StepArgs<T> &a, const SegCtx<T> &s, int g, const T (&dx)[5],
+                                            const T (&dy)[5], const T (&dz)[5], T (&un)[5]) {
+  new_state(a, s, g, dx, dy, dz, un);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) a.U[v * a.S + g] = un[v];
+}
+
+// father cell (index in its oct) of the oct with internal key k
+__device__ __forceinline__ int father_cell(uint64_t k) {
+  return int((ikey_x(k) & 1) | ((ikey_y(k) & 1) << 1) | ((ikey_z(k) & 1) << 2));
+}
+
+// The last pass of a level step: update(s, t, u) gives local cell t's new state
+// (stored in U by it, or the standing one of a split cell); then, from the same
+// warp's values, the restriction of its octs onto their father cells, (sum of
+// the 8 children in child order) / 8, and (REFLUX) beyond the cells the reflux
+// sums of the level's ghost octs.  They touch disjoint data: the level's cells,
+// the coarser level's split cells, the pending reflux of its leaf cells.
+// domain: 8 nl, + 5 ncl (if REFLUX and kSegReflux)
+template <class T, bool REFLUX, class Update>
+__device__ __forceinline__ void update_loop(const StepArgs<T> &a, Update update) {
+  extern __shared__ __align__(8) unsigned char update_smem[];  // the block's new states [5][threads]
+  T *sm = reinterpret_cast<T *>(update_smem);
+  const int lane = threadIdx.x & 31;
+  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tiles, ti);
+    const Seg sg = seg_at(a.tiles, td.seg);
+    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
+    const SegCtx<T> s = seg_ctx(a, sg);
+#ifdef AMR_CHECKED
+    if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
+      atomicOr(a.err, kErrIndex);
+      continue;
+    }
+#endif
+    const int t = td.start + threadIdx.x;
+    if (t < 8 * s.nl) {
+      T u[5];
+      update(s, t, u);
+      if (s.flags & kSegRestrict) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) sm[v * blockDim.x + threadIdx.x] = u[v];
+      }
+    } else if (REFLUX && (s.flags & kSegReflux) && t - 8 * s.nl < 5 * s.ncl) {
+      const int q = t - 8 * s.nl, v = q / s.ncl;
+      reflux_sum(a, v, s.clo + (q - v * s.ncl));
+    }
+    if (s.flags & kSegRestrict) {
+      __syncwarp();
+      const int q = ((t - lane) >> 3) + (lane & 3), v = lane >> 2;  // local oct, variable
+      if (v < 5 && q < s.nl) {
+        const int o = s.lo + q;
+        const int fc = father_cell(__ldg(a.key + o));
+        const int f = int(checked(__ldg(a.father + o), 0, a.N, a.err));
+        const T *src = sm + v * blockDim.x + (threadIdx.x - lane) + 8 * (lane & 3);
+        T sum = T(0);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) sum += src[c];
+        a.U[v * a.S + 8 * int64_t(f) + fc] = sum * T(0.125);
+      }
+      __syncwarp();
+    }
   }
 }
 
-template <class T>
-__device__ __forceinline__ void update_cell(const StepArgs<T> &a, const SegCtx<T> &s, int g,
-                                            const T (&dx)[5], const T (&dy)[5], const T (&dz)[5]) {
-  update_cell_to(a, s, g, dx, dy, dz, a.U + g, a.S);
-}
-
-template <class T>
-__global__ void k_update(StepArgs<T> a) {
-  tile_loop(a, [](const SegCtx<T> &s) { return 8 * s.nl; }, [&](const SegCtx<T> &s, int t) {
-    if (cell_is_split(a, s, t)) return;
+__global__ void __launch_bounds__(512, 3) k_update(StepArgs<double> a) {
+  update_loop<double, true>(a, [&](const SegCtx<double> &s, int t, double (&u)[5]) {
     const int e = s.lo + (t >> 3);
     const int c = t & 7;
+    if (cell_is_split(a, s, t)) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + 8 * e + c];
+      return;
+    }
     const int o = s.base + t;
     const int om[3] = {s.base + nbr_local(a, s, t, e, c, 0, 0), s.base + nbr_local(a, s, t, e, c, 1, 0),
                        s.base + nbr_local(a, s, t, e, c, 2, 0)};
-    T dx[5], dy[5], dz[5];
+    double dx[5], dy[5], dz[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       dx[v] = a.F[(0 + v) * a.LS + om[0]] - a.F[(0 + v) * a.LS + o];
       dy[v] = a.F[(5 + v) * a.LS + om[1]] - a.F[(5 + v) * a.LS + o];
       dz[v] = a.F[(10 + v) * a.LS + om[2]] - a.F[(10 + v) * a.LS + o];
     }
-    update_cell(a, s, 8 * e + c, dx, dy, dz);
+    update_cell(a, s, 8 * e + c, dx, dy, dz, u);
   });
 }
 
@@ -774,49 +923,32 @@ __device__ __forceinline__ void faces_dir(const StepArgs<T> &a, const SegCtx<T> 
   for (int v = 0; v < 5; ++v) du[v] = Fm[v] - Fp[v];
 }
 
-template <class T>
-__global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<T> a) {
-  tile_loop(a, [](const SegCtx<T> &s) { return 8 * s.nl; }, [&](const SegCtx<T> &s, int t) {
-    if (cell_is_split(a, s, t)) return;
+__global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<float> a) {
+  update_loop<float, false>(a, [&](const SegCtx<float> &s, int t, float (&u)[5]) {
     const int e = s.lo + (t >> 3);
     const int c = t & 7;
-    T dx[5], dy[5], dz[5];
+    if (cell_is_split(a, s, t)) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + 8 * e + c];
+      return;
+    }
+    float dx[5], dy[5], dz[5];
     faces_dir<0>(a, s, t, e, c, dx);
     faces_dir<1>(a, s, t, e, c, dy);
     faces_dir<2>(a, s, t, e, c, dz);
-    update_cell(a, s, 8 * e + c, dx, dy, dz);
+    update_cell(a, s, 8 * e + c, dx, dy, dz, u);
   });
 }
 
-// Reflux: R(X) += sum of the 24 slots of the ghost oct whose father is X, in
-// slot order (direction -x,+x,-y,+y,-z,+z seen from X, then fine face).
-// Restriction: father cell = (sum of the 8 children in child order) / 8.
-// They touch disjoint data (leaf cells' pending reflux, split cells).
-// domain: 5 ncl (if kSegReflux) + 5 nl (if kSegRestrict)
+// Restriction alone (of a state that was written): father cell = (sum of the 8
+// children in child order) / 8.  domain: 5 nl (if kSegRestrict)
 template <class T>
-__global__ void k_reflux_restrict(StepArgs<T> a) {
-  tile_loop(a,
-            [](const SegCtx<T> &s) {
-              return ((s.flags & kSegReflux) ? 5 * s.ncl : 0) + ((s.flags & kSegRestrict) ? 5 * s.nl : 0);
-            },
-            [&](const SegCtx<T> &s, int q) {
-              const int nref = (s.flags & kSegReflux) ? 5 * s.ncl : 0;
-              if (q < nref) {
-                const int v = q / s.ncl;
-                const int g = s.clo + (q - v * s.ncl);
-                const T *cv = a.C + v * a.CS + 24 * int64_t(g);
-                T *Rv = a.Rc + v * int64_t(a.NC) + g;
-                T acc = *Rv;
-#pragma unroll
-                for (int k = 0; k < 24; ++k) acc += cv[k];
-                *Rv = acc;
-                return;
-              }
-              const int r = q - nref;
+__global__ void k_restrict(StepArgs<T> a) {
+  tile_loop(a, [](const SegCtx<T> &s) { return (s.flags & kSegRestrict) ? 5 * s.nl : 0; },
+            [&](const SegCtx<T> &s, int r) {
               const int v = r / s.nl;
               const int o = s.lo + (r - v * s.nl);
-              const uint64_t k = __ldg(a.key + o);
-              const int fc = int((ikey_x(k) & 1) | ((ikey_y(k) & 1) << 1) | ((ikey_z(k) & 1) << 2));
+              const int fc = father_cell(__ldg(a.key + o));
               const int f = int(checked(__ldg(a.father + o), 0, a.N, a.err));
               const T *src = a.U + v * a.S + 8 * int64_t(o);
               T sum = T(0);
@@ -845,7 +977,7 @@ __device__ __forceinline__ void cfl_flush(const CflArgs &a, double s, int seg, d
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s = fmax(s, __shfl_xor_sync(0xFFFFFFFFu, s, off));
     if (lane == 0 && s > 0.0) {
-      const Seg sg = a.segs[seg];
+      const Seg sg = seg_at(a.tiles, seg);
       atomicMax(a.smax + 16 * sg.member + sg.level, (unsigned long long)__double_as_longlong(s));
     }
   }
@@ -875,14 +1007,14 @@ __global__ void k_cfl_fp32(CflArgs a, const float *U) {
   int cur = -1;
   const float *mgamma = static_cast<const float *>(a.mgamma_t), *msmallr = static_cast<const float *>(a.msmallr_t),
               *msmallp = static_cast<const float *>(a.msmallp_t);
-  for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tpre, a.tseg0, a.tnseg, a.tstep, ti);
+  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tiles, ti);
     if (td.seg != cur) {
       if (cur >= 0) cfl_flush<float>(a, double(s), cur, wmax);
       s = 0.0f;
       cur = td.seg;
     }
-    const Seg sg = a.segs[td.seg];
+    const Seg sg = seg_at(a.tiles, td.seg);
     const int t = td.start + threadIdx.x;
     if (t < 8 * sg.nl && a.mrem[sg.member] != 0 &&
         !((__ldg(a.son + sg.lo + (t >> 3)) >> (t & 7)) & 1u)) {
@@ -920,9 +1052,9 @@ __global__ void k_cfl_fp32(CflArgs a, const float *U) {
 // momentum makes its kinetic energy so.
 __global__ void __launch_bounds__(512) k_cfl_fp64(CflArgs a, const double *U) {
   const double *mgamma = a.mgamma, *msmallr = a.msmallr, *msmallp = a.msmallp;
-  for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tpre, a.tseg0, a.tnseg, a.tstep, ti);
-    const Seg sg = a.segs[td.seg];
+  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tiles, ti);
+    const Seg sg = seg_at(a.tiles, td.seg);
     const int t = td.start + threadIdx.x;
     unsigned long long *out = a.smax + 16 * sg.member + sg.level;
     bool test = false;

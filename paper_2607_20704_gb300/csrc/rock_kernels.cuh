@@ -214,11 +214,11 @@ __global__ void __launch_bounds__(Rock<NS>::THREADS, Rock<NS>::template min_bloc
 
   for (int q = t; q < NB; q += TH) pos_oct[q] = -1;
   __syncthreads();
-  for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tpre, a.tseg0, a.tnseg, a.tstep, ti);
-    const Seg sg = a.segs[td.seg];
+  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tiles, ti);
+    const Seg sg = seg_at(a.tiles, td.seg);
     if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member (block-uniform)
-    const SegCtx<T> s = seg_ctx(a, td.seg);
+    const SegCtx<T> s = seg_ctx(a, sg);
     const int gb = sg.blk0 + td.start;
     const int o0 = int(checked(__ldg(blk + gb), s.lo, s.lo + s.nl, a.err, s.lo));
     const int o1 = int(checked(__ldg(blk + gb + 1), o0 + 1, s.lo + s.nl + 1, a.err, o0 + 1));
@@ -455,8 +455,7 @@ __global__ void __launch_bounds__(Rock<NS>::THREADS, Rock<NS>::template min_bloc
 
 // After a fused kernel: the new states of the level's leaf cells from the
 // scratch W into U, the reflux sums of the level's ghost octs and the
-// restriction onto the father cells (what k_reflux_restrict does after the
-// per-cell passes, with the commit folded in).  Thread per (oct, variable):
+// restriction onto the father cells (as the last per-cell pass does).  Thread per (oct, variable):
 // 8 values in, 8 out, the restriction from the same 8 values.
 // domain: 5 ncl (if kSegReflux) + 5 nl
 template <class T>
@@ -467,13 +466,7 @@ __global__ void k_commit_post(StepArgs<T> a) {
               const int nref = (s.flags & kSegReflux) ? 5 * s.ncl : 0;
               if (q < nref) {
                 const int v = q / s.ncl;
-                const int g = s.clo + (q - v * s.ncl);
-                const T *cv = a.C + v * a.CS + 24 * int64_t(g);
-                T *Rv = a.Rc + v * int64_t(a.NC) + g;
-                T acc = *Rv;
-#pragma unroll
-                for (int k = 0; k < 24; ++k) acc += cv[k];
-                *Rv = acc;
+                reflux_sum(a, v, s.clo + (q - v * s.ncl));
                 return;
               }
               const int r = q - nref;
@@ -491,8 +484,7 @@ __global__ void k_commit_post(StepArgs<T> a) {
               }
               store_oct8(u, val);
               if (s.flags & kSegRestrict) {
-                const uint64_t k = __ldg(a.key + o);
-                const int fc = int((ikey_x(k) & 1) | ((ikey_y(k) & 1) << 1) | ((ikey_z(k) & 1) << 2));
+                const int fc = father_cell(__ldg(a.key + o));
                 const int f = int(checked(__ldg(a.father + o), 0, a.N, a.err));
                 T sum = T(0);
 #pragma unroll
@@ -548,11 +540,11 @@ __global__ void __launch_bounds__(Sweep<NS>::THREADS) k_sweep(StepArgs<T> a, con
   constexpr int E = R::E, P = R::P, NO = R::NO, QE = R::QE, QP = R::QP, IN = R::IN, FP = R::FP,
                 ZF = R::ZF, FNP = R::FNP, TH = R::THREADS;
 
-  for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tpre, a.tseg0, a.tnseg, a.tstep, ti);
-    const Seg sg = a.segs[td.seg];
+  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
+    const Tile td = tile_at(a.tiles, ti);
+    const Seg sg = seg_at(a.tiles, td.seg);
     if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member (block-uniform)
-    const SegCtx<T> s = seg_ctx(a, td.seg);
+    const SegCtx<T> s = seg_ctx(a, sg);
     const int gb = sg.blk0 + td.start;
     const int o0 = int(checked(__ldg(blk + gb), s.lo, s.lo + s.nl, a.err, s.lo));
     const int o1 = int(checked(__ldg(blk + gb + 1), o0 + 1, s.lo + s.nl + 1, a.err, o0 + 1));
@@ -681,7 +673,10 @@ __global__ void __launch_bounds__(Sweep<NS>::THREADS) k_sweep(StepArgs<T> a, con
               du[2][v] = Fzl[v * ZF + (x - 2) + IN * (y - 2)] - Fzc[v * ZF + (x - 2) + IN * (y - 2)];
             }
             const int t = 8 * (e - s.lo) + c;
-            update_cell_to(a, s, 8 * e + c, du[0], du[1], du[2], a.W + s.base + t, int64_t(a.LS));
+            T un[5];  // into the scratch: other blocks may still read the old state
+            new_state(a, s, 8 * e + c, du[0], du[1], du[2], un);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) a.W[v * int64_t(a.LS) + s.base + t] = un[v];
           }
         }
         __syncthreads();
