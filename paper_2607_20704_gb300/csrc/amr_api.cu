@@ -296,6 +296,20 @@ struct amr_mesh {
   int64_t steps_on_mesh = 0;  // coarse steps since this mesh was built
   cudaGraphExec_t graph = nullptr;
   int64_t graph_kernels = 0;
+  // the launches of a Poisson solve (hundreds of small ones), captured at the
+  // second call with the same arguments on this mesh
+  struct PoissonCall {
+    int member = -1, n_vcycles = 0;
+    bool levels = false;
+    double fourpiG = 0.0;
+    bool operator==(const PoissonCall &o) const {
+      return member == o.member && n_vcycles == o.n_vcycles && levels == o.levels &&
+             std::memcmp(&fourpiG, &o.fourpiG, sizeof fourpiG) == 0;
+    }
+  };
+  PoissonCall poisson_call;  // the last call's arguments
+  cudaGraphExec_t poisson_graph = nullptr;
+  int64_t poisson_kernels = 0;
   bool timing = false;
   std::vector<TimedLaunch> pending;
   std::vector<cudaEvent_t> event_pool;
@@ -1072,6 +1086,7 @@ static void destroy_all(amr_mesh *h) {
   if (h->cs) cudaStreamDestroy(h->cs);
   if (h->cs_out) cudaStreamDestroy(h->cs_out);
   if (h->graph) cudaGraphExecDestroy(h->graph);
+  if (h->poisson_graph) cudaGraphExecDestroy(h->poisson_graph);
   for (auto &t : h->pending) {
     cudaEventDestroy(t.e0);
     cudaEventDestroy(t.e1);
@@ -2352,8 +2367,16 @@ extern "C" amr_status amr_regrid_flags(amr_handle h, const uint8_t *flags, int64
 constexpr int kMGParts = 1024;  // blocks of the reductions
 constexpr int kMGPre = 2, kMGPost = 2, kMGCoarsest = 8;
 
+// arrays that the captured solve reads are about to be replaced
+static void drop_poisson_graph(amr_mesh *h) {
+  if (h->poisson_graph) cudaGraphExecDestroy(h->poisson_graph);
+  h->poisson_graph = nullptr;
+  h->poisson_call = amr_mesh::PoissonCall();
+}
+
 static amr_status mg_setup(amr_mesh *h, int member, int lmin) {
   if (h->mg_member == member && !h->mg.empty() && h->mg[0].n == (1 << lmin)) return AMR_OK;
+  drop_poisson_graph(h);
   for (auto &L : h->mg) {
     dev_free(h, L.f);
     dev_free(h, L.p);
@@ -2386,39 +2409,46 @@ static unsigned mg_blocks(int64_t m) { return unsigned(std::min<int64_t>((m + 25
 
 static void mg_vcycle(amr_mesh *h, size_t k, double dx) {
   amr_mesh::MGLevel &L = h->mg[k];
-  const int n = L.n;
+  const int n = L.n, b = bits_for(n);
   const double dx2 = dx * dx;
-  if (n <= 2) {
-    launch(h, K_MG_OTHER, k_mg_coarsest, dim3(1), dim3(8), dx2, (const double *)L.f, L.p, kMGCoarsest);
+  if (n <= kMGTail) {
+    launch(h, K_MG_OTHER, k_mg_tail, dim3(1), dim3(256), b, dx2, (const double *)L.f, L.p, kMGPre, kMGPost,
+           kMGCoarsest);
     return;
   }
   const int64_t m = int64_t(n) * n * n;
   for (int s = 0; s < kMGPre; ++s)
     for (int colour = 0; colour < 2; ++colour)
-      launch(h, K_MG_SMOOTH, k_mg_smooth, dim3(nblocks(m / 2)), dim3(256), n, dx2, (const double *)L.f,
+      launch(h, K_MG_SMOOTH, k_mg_smooth, dim3(nblocks(m / 2)), dim3(256), b, dx2, (const double *)L.f,
              L.p, colour);
   amr_mesh::MGLevel &C = h->mg[k + 1];
-  launch(h, K_MG_RESTRICT, k_mg_restrict, dim3(nblocks(m / 8)), dim3(256), n, 1.0 / dx2,
+  launch(h, K_MG_RESTRICT, k_mg_restrict, dim3(nblocks(m / 8, 64)), dim3(64), b, 1.0 / dx2,
          (const double *)L.f, (const double *)L.p, C.f, C.p);
   mg_vcycle(h, k + 1, 2.0 * dx);
-  launch(h, K_MG_PROLONG, k_mg_prolong, dim3(nblocks(m)), dim3(256), n, (const double *)C.p, L.p);
+  launch(h, K_MG_PROLONG, k_mg_prolong, dim3(nblocks(m / 8, 64)), dim3(64), b, (const double *)C.p, L.p);
   for (int s = 0; s < kMGPost; ++s)
     for (int colour = 0; colour < 2; ++colour)
-      launch(h, K_MG_SMOOTH, k_mg_smooth, dim3(nblocks(m / 2)), dim3(256), n, dx2, (const double *)L.f,
+      launch(h, K_MG_SMOOTH, k_mg_smooth, dim3(nblocks(m / 2)), dim3(256), b, dx2, (const double *)L.f,
              L.p, colour);
 }
 
-extern "C" amr_status amr_poisson(amr_handle h, double fourpiG, int n_vcycles, double *resid) {
-  if (!h) return fail(AMR_EINVAL, "amr_poisson: NULL handle");
+// arguments and buffers of a base-level solve
+static amr_status poisson_setup(amr_mesh *h, int n_vcycles) {
   if (n_vcycles < 0 || n_vcycles > 1020) return fail(AMR_EINVAL, "amr_poisson: n_vcycles must be in [0, 1020]");
   const Member &mb = h->mem[h->sel];
   const int lmin = mb.lmin;
   if (lmin > 10) return fail(AMR_EINVAL, "amr_poisson: levelmin above 10 (more than 1024^3 cells)");
-  const int n = 1 << lmin;
+  if (8 * (mb.lo[lmin + 1] - mb.lo[lmin]) != int64_t(1) << (3 * lmin))
+    return fail(AMR_EGRADING, "amr_poisson: the base level is not complete");
+  return mg_setup(h, h->sel, lmin);
+}
+
+// the launches of a base-level solve
+static void poisson_base(amr_mesh *h, double fourpiG, int n_vcycles, bool resid) {
+  const Member &mb = h->mem[h->sel];
+  const int lmin = mb.lmin, n = 1 << lmin;
   const int64_t m0 = int64_t(n) * n * n;
   const int lo = int(mb.oct_base + mb.lo[lmin]), nl = int(mb.lo[lmin + 1] - mb.lo[lmin]);
-  if (8 * int64_t(nl) != m0) return fail(AMR_EGRADING, "amr_poisson: the base level is not complete");
-  AMR_TRY(mg_setup(h, h->sel, lmin));
   const double dx = std::ldexp(1.0, -lmin);
   if (h->p.precision == 4)
     launch(h, K_MG_OTHER, k_mg_gather<float>, dim3(nblocks(m0)), dim3(256), (const float *)h->U,
@@ -2450,8 +2480,59 @@ extern "C" amr_status amr_poisson(amr_handle h, double fourpiG, int n_vcycles, d
          int(nb), 1.0 / double(m0), mean + 1);
   launch(h, K_MG_OTHER, k_mg_scatter, dim3(nblocks(m0)), dim3(256), (const double *)h->mg[0].p,
          (const uint64_t *)h->key, lo, nl, n, (const double *)(mean + 1), h->phi);
-  if (resid && n_vcycles > 0)
-    CUDA_TRY(cudaMemcpyAsync(resid, h->mg_res, sizeof(double) * n_vcycles, cudaMemcpyDeviceToHost, h->s));
+}
+
+// run `solve` (the launches of one call without residual norms): directly the
+// first time, replayed as a CUDA graph from the second call with the same
+// arguments on (the first launch of a solve on a new mesh is not delayed by a
+// capture)
+template <class Solve>
+static amr_status poisson_run(amr_mesh *h, const amr_mesh::PoissonCall &call, Solve solve) {
+  if (!h->p.use_graphs || h->timing) return solve();
+  if (!(h->poisson_call == call)) {
+    drop_poisson_graph(h);
+    h->poisson_call = call;
+    return solve();
+  }
+  if (!h->poisson_graph) {
+    h->capturing = true;
+    h->capture_kernels = 0;
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(h->s, cudaStreamCaptureModeThreadLocal);
+    amr_status st = AMR_OK;
+    if (e == cudaSuccess) {
+      st = solve();
+      e = cudaStreamEndCapture(h->s, &g);
+    }
+    h->capturing = false;
+    if (e == cudaSuccess && st == AMR_OK) e = cudaGraphInstantiate(&h->poisson_graph, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess || st != AMR_OK) {  // e.g. a stream that cannot be captured: launch directly
+      cudaGetLastError();
+      h->poisson_graph = nullptr;
+      return solve();
+    }
+    h->poisson_kernels = h->capture_kernels;
+  }
+  CUDA_TRY(cudaGraphLaunch(h->poisson_graph, h->s));
+  h->graph_launches++;
+  h->launches += h->poisson_kernels;
+  return AMR_OK;
+}
+
+extern "C" amr_status amr_poisson(amr_handle h, double fourpiG, int n_vcycles, double *resid) {
+  if (!h) return fail(AMR_EINVAL, "amr_poisson: NULL handle");
+  AMR_TRY(poisson_setup(h, n_vcycles));
+  if (resid) {
+    poisson_base(h, fourpiG, n_vcycles, true);
+    if (n_vcycles > 0)
+      CUDA_TRY(cudaMemcpyAsync(resid, h->mg_res, sizeof(double) * n_vcycles, cudaMemcpyDeviceToHost, h->s));
+  } else {
+    AMR_TRY(poisson_run(h, {h->sel, n_vcycles, false, fourpiG}, [&] {
+      poisson_base(h, fourpiG, n_vcycles, false);
+      return AMR_OK;
+    }));
+  }
   return check_device(h, "amr_poisson");
 }
 
@@ -2460,6 +2541,7 @@ extern "C" amr_status amr_poisson(amr_handle h, double fourpiG, int n_vcycles, d
 // ---------------------------------------------------------------------------
 static amr_status ensure_phil(amr_mesh *h) {
   if (h->phil && h->phil_n == 8 * h->N) return AMR_OK;
+  drop_poisson_graph(h);
   dev_free(h, h->phil);
   h->phil = nullptr;
   AMR_TRY(alloc_n(h, &h->phil, 8 * std::max<int64_t>(h->N, 1)));
@@ -2632,33 +2714,39 @@ static amr_status mgl_setup(amr_mesh *h, int L, amr_mesh::MGLSet **out) {
   return AMR_OK;
 }
 
-static void mgl_sweep(amr_mesh *h, amr_mesh::MGLSet &S, size_t k) {
+static void mgl_sweeps(amr_mesh *h, amr_mesh::MGLSet &S, size_t k, int sweeps) {
   amr_mesh::MGLTab &T = S.tab[k];
   const double dx = std::ldexp(1.0, -T.L), dx2 = dx * dx;
   const double *bs = k == 0 ? S.bsum : nullptr;
-  if (T.nc0)
-    launch(h, K_MG_SMOOTH, k_mgl_smooth, dim3(nblocks(T.nc0)), dim3(256), T.n, (const int32_t *)T.col, T.nc0,
-           (const int32_t *)T.nb, (const int32_t *)T.nbnd, bs, (const double *)T.f, T.e, dx2);
-  if (T.nc1)
-    launch(h, K_MG_SMOOTH, k_mgl_smooth, dim3(nblocks(T.nc1)), dim3(256), T.n, (const int32_t *)(T.col + T.nc0),
-           T.nc1, (const int32_t *)T.nb, (const int32_t *)T.nbnd, bs, (const double *)T.f, T.e, dx2);
+  if (T.n <= kMGLBlock) {
+    launch(h, K_MG_SMOOTH, k_mgl_sweeps, dim3(1), dim3(512), T.n, (const int32_t *)T.col, T.nc0,
+           (const int32_t *)T.nb, (const int32_t *)T.nbnd, bs, (const double *)T.f, T.e, dx2, sweeps);
+    return;
+  }
+  for (int s = 0; s < sweeps; ++s) {
+    if (T.nc0)
+      launch(h, K_MG_SMOOTH, k_mgl_smooth, dim3(nblocks(T.nc0)), dim3(256), T.n, (const int32_t *)T.col, T.nc0,
+             (const int32_t *)T.nb, (const int32_t *)T.nbnd, bs, (const double *)T.f, T.e, dx2);
+    if (T.nc1)
+      launch(h, K_MG_SMOOTH, k_mgl_smooth, dim3(nblocks(T.nc1)), dim3(256), T.n, (const int32_t *)(T.col + T.nc0),
+             T.nc1, (const int32_t *)T.nb, (const int32_t *)T.nbnd, bs, (const double *)T.f, T.e, dx2);
+  }
 }
 
 static void mgl_residual(amr_mesh *h, amr_mesh::MGLSet &S, size_t k) {
   amr_mesh::MGLTab &T = S.tab[k];
-  const double dx = std::ldexp(1.0, -T.L), dx2 = dx * dx;
   launch(h, K_MG_OTHER, k_mgl_residual, dim3(nblocks(T.n)), dim3(256), T.n, (const int32_t *)T.nb,
          (const int32_t *)T.nbnd, (const double *)(k == 0 ? S.bsum : nullptr), (const double *)T.f,
-         (const double *)T.e, dx2, T.r);
+         (const double *)T.e, std::ldexp(1.0, 2 * T.L), T.r);
 }
 
 static void mgl_vcycle(amr_mesh *h, amr_mesh::MGLSet &S, size_t k) {
   const size_t K = S.tab.size() - 1;
   if (k == K) {
-    for (int s = 0; s < kMGCoarsest; ++s) mgl_sweep(h, S, k);
+    mgl_sweeps(h, S, k, kMGCoarsest);
     return;
   }
-  for (int s = 0; s < kMGPre; ++s) mgl_sweep(h, S, k);
+  mgl_sweeps(h, S, k, kMGPre);
   mgl_residual(h, S, k);
   amr_mesh::MGLTab &T = S.tab[k], &C = S.tab[k + 1];
   launch(h, K_MG_RESTRICT, k_mgl_restrict, dim3(nblocks(C.n)), dim3(256), C.n, (const int32_t *)C.child,
@@ -2666,7 +2754,7 @@ static void mgl_vcycle(amr_mesh *h, amr_mesh::MGLSet &S, size_t k) {
   mgl_vcycle(h, S, k + 1);
   launch(h, K_MG_PROLONG, k_mgl_prolong, dim3(nblocks(T.n)), dim3(256), T.n, (const int32_t *)T.pro,
          (const double *)C.e, T.e);
-  for (int s = 0; s < kMGPost; ++s) mgl_sweep(h, S, k);
+  mgl_sweeps(h, S, k, kMGPost);
 }
 
 // one level's solve from the current potential of level L-1 (Dirichlet
@@ -2735,21 +2823,36 @@ __global__ void k_mgl_inject(int lo, int nl, const uint64_t *__restrict__ key, c
 extern "C" amr_status amr_poisson_levels(amr_handle h, double fourpiG, int n_vcycles, double *resid) {
   if (!h) return fail(AMR_EINVAL, "amr_poisson_levels: NULL handle");
   const Member &mb = h->mem[h->sel];
-  std::vector<double> r0(size_t(std::max(n_vcycles, 1)));
-  AMR_TRY(amr_poisson(h, fourpiG, n_vcycles, resid ? r0.data() : nullptr));
+  AMR_TRY(poisson_setup(h, n_vcycles));
   AMR_TRY(ensure_phil(h));
+  int top = mb.lmin;  // the finest populated level; the hierarchies' tables exist before the launches
+  for (; top < mb.lmax && mb.lo[top + 2] > mb.lo[top + 1]; ++top) {
+    amr_mesh::MGLSet *S = nullptr;
+    AMR_TRY(mgl_setup(h, top + 1, &S));
+  }
   const int64_t blo = mb.oct_base + mb.lo[mb.lmin], bnl = mb.lo[mb.lmin + 1] - mb.lo[mb.lmin];
-  CUDA_TRY(cudaMemcpyAsync(h->phil + 8 * blo, h->phi, sizeof(double) * size_t(8 * bnl), cudaMemcpyDeviceToDevice, h->s));
-  if (resid)
+  const double *mean = h->mg_res + 1022;  // the base density's mean (poisson_base)
+  auto refined = [&]() -> amr_status {
+    CUDA_TRY(cudaMemcpyAsync(h->phil + 8 * blo, h->phi, sizeof(double) * size_t(8 * bnl), cudaMemcpyDeviceToDevice,
+                             h->s));
+    for (int L = mb.lmin + 1; L <= top; ++L) {
+      const int lo = int(mb.oct_base + mb.lo[L]), nl = int(mb.lo[L + 1] - mb.lo[L]);
+      launch(h, K_MG_OTHER, k_mgl_inject, dim3(nblocks(8 * int64_t(nl))), dim3(256), lo, nl,
+             (const uint64_t *)h->key, (const int32_t *)h->father, h->phil);
+      AMR_TRY(poisson_level(h, L, fourpiG, 0.0, mean, n_vcycles, resid ? resid + size_t(L) * n_vcycles : nullptr));
+    }
+    return AMR_OK;
+  };
+  if (resid) {
+    std::vector<double> r0(size_t(std::max(n_vcycles, 1)));
+    AMR_TRY(amr_poisson(h, fourpiG, n_vcycles, r0.data()));
     for (int c = 0; c < n_vcycles; ++c) resid[size_t(mb.lmin) * n_vcycles + c] = r0[size_t(c)];
-  const double *mean = h->mg_res + 1022;  // the base density's mean (amr_poisson)
-  for (int L = mb.lmin + 1; L <= mb.lmax; ++L) {
-    const int lo = int(mb.oct_base + mb.lo[L]), nl = int(mb.lo[L + 1] - mb.lo[L]);
-    if (nl == 0) break;
-    launch(h, K_MG_OTHER, k_mgl_inject, dim3(nblocks(8 * int64_t(nl))), dim3(256), lo, nl,
-           (const uint64_t *)h->key, (const int32_t *)h->father, h->phil);
-    AMR_TRY(poisson_level(h, L, fourpiG, 0.0, mean, n_vcycles,
-                          resid ? resid + size_t(L) * n_vcycles : nullptr));
+    AMR_TRY(refined());
+  } else {
+    AMR_TRY(poisson_run(h, {h->sel, n_vcycles, true, fourpiG}, [&] {
+      poisson_base(h, fourpiG, n_vcycles, false);
+      return refined();
+    }));
   }
   return check_device(h, "amr_poisson_levels");
 }

@@ -12,13 +12,15 @@
 // The base level lives in the mesh's oct order; the solver works on dense
 // arrays [x + n (y + n z)] of every multigrid level (unit-stride x, so every
 // stencil access is coalesced), gathered from and scattered back to the octs.
-// On GB300 the FP64 pipe bounds these stencils (about 8 FP64 operations per
-// cell against 16 bytes of traffic); no step divides: the Gauss-Seidel update
-// multiplies by the rounded 1/6 where the operator divides by 6 (the two differ
-// by at most a few units in the last place per update), and the residual
-// multiplies by 1/dx^2, which is exact (dx is a power of two).
+// On GB300 the FP64 pipe bounds these stencils on the large grids (7 FP64
+// operations per smoothed cell against 16 bytes of traffic) and the launches on
+// the small ones; no step divides: the Gauss-Seidel update multiplies by the
+// rounded 1/6 where the operator divides by 6 (the two differ by at most a few
+// units in the last place per update; the product runs on the integer pipes),
+// and the residual multiplies by 1/dx^2, which is exact (dx is a power of two).
 #pragma once
 #include "amr_internal.cuh"
+#include "fp64_int.cuh"
 
 namespace amr {
 
@@ -65,13 +67,21 @@ __global__ void k_mg_sum(const double *__restrict__ a, int64_t m, int sq, double
   }
 }
 
-// out = scale * (sum of the partial sums); one thread
+// sum of the partial sums by one warp: lane l adds parts l, l + 32, .., then a
+// fixed butterfly (one thread adding up to 1024 of them in turn took 20 us)
+__device__ __forceinline__ double mg_sum_parts(const double *__restrict__ part, int nparts) {
+  double s = 0.0;
+  for (int q = threadIdx.x; q < nparts; q += 32) s += part[q];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+  return s;
+}
+
+// out = scale * (sum of the partial sums); one warp
 __global__ void k_mg_total(const double *__restrict__ part, int nparts, double scale,
                            double *__restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0.0;
-  for (int q = 0; q < nparts; ++q) s += part[q];
-  *out = s * scale;
+  const double s = mg_sum_parts(part, nparts);
+  if (threadIdx.x == 0) *out = s * scale;
 }
 
 // f = fourpiG (rho - mean)
@@ -82,67 +92,158 @@ __global__ void k_mg_source(const double *__restrict__ rho, int64_t m, const dou
     f[t] = fourpiG * (rho[t] - mu);
 }
 
-// one colour of a red-black sweep: thread t -> (x, y, z) with x + y + z of
-// the colour's parity
-__global__ void k_mg_smooth(int n, double dx2, const double *__restrict__ f, double *p, int colour) {
-  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  const int64_t half = int64_t(n) * n * n / 2;
-  if (t >= half) return;
-  const int h = n >> 1;
-  const int xh = int(t % h);
-  const int64_t yz = t / h;
-  const int y = int(yz % n), z = int(yz / n);
-  const int x = 2 * xh + ((y + z + colour) & 1);
-  const int64_t i = mg_at(n, x, y, z);
-  p[i] = (mg_nbsum(n, p, x, y, z) - dx2 * f[i]) * (1.0 / 6.0);
+// v / 6 as v times the rounded 1/6, on the integer pipes (NaN, infinities and
+// values near overflow: on the FP64 pipe)
+__device__ __forceinline__ double mg_sixth(double v) {
+  return below<1000>(v) ? mul_int0(v, 1.0 / 6.0) : v * (1.0 / 6.0);
 }
 
-// coarse source = mean of the 8 children's residuals; coarse correction = 0
-__global__ void k_mg_restrict(int n, double inv_dx2, const double *__restrict__ f,
-                              const double *__restrict__ p, double *__restrict__ fc, double *__restrict__ ec) {
-  const int h = n >> 1;
-  const int64_t T = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (T >= int64_t(h) * h * h) return;
-  const int X = int(T % h), Y = int((T / h) % h), Z = int(T / (int64_t(h) * h));
-  double s = 0.0;
+// one colour of a red-black sweep: thread t -> (x, y, z) with x + y + z of
+// the colour's parity; n = 2^b
+__global__ void k_mg_smooth(int b, double dx2, const double *__restrict__ f, double *p, int colour) {
+  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (t >= int64_t(1) << (3 * b - 1)) return;
+  const int n = 1 << b;
+  const int64_t yz = t >> (b - 1);
+  const int y = int(yz) & (n - 1), z = int(yz >> b);
+  const int x = 2 * (int(t) & (n / 2 - 1)) + ((y + z + colour) & 1);
+  const int64_t i = mg_at(n, x, y, z);
+  p[i] = mg_sixth(mg_nbsum(n, p, x, y, z) - dx2 * f[i]);
+}
+
+// coarse source = mean of the 8 children's residuals; coarse correction = 0.
+// Three of a child's neighbours lie in the block of 8 and cancel against half
+// of its diagonal when the residuals are summed: the sum needs, per child, its
+// three outer neighbours less 3 p (39 FP64 operations per block, 72 with eight
+// residuals).
+__device__ __forceinline__ double mg_block_residual(int n, double inv_dx2, const double *__restrict__ f,
+                                                    const double *__restrict__ p, int X, int Y, int Z) {
+  double sf = 0.0, sp = 0.0;
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const int x = 2 * X + (c & 1), y = 2 * Y + ((c >> 1) & 1), z = 2 * Z + ((c >> 2) & 1);
+    const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
+    const int x = 2 * X + cx, y = 2 * Y + cy, z = 2 * Z + cz;
     const int64_t i = mg_at(n, x, y, z);
-    s += f[i] - (mg_nbsum(n, p, x, y, z) - 6.0 * p[i]) * inv_dx2;
+    sf += f[i];
+    sp += ((p[mg_at(n, x + 2 * cx - 1, y, z)] + p[mg_at(n, x, y + 2 * cy - 1, z)]) +
+           p[mg_at(n, x, y, z + 2 * cz - 1)]) - 3.0 * p[i];
   }
-  fc[T] = s * 0.125;
+  return (sf - sp * inv_dx2) * 0.125;
+}
+__global__ void k_mg_restrict(int b, double inv_dx2, const double *__restrict__ f,
+                              const double *__restrict__ p, double *__restrict__ fc, double *__restrict__ ec) {
+  const int64_t T = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  const int bc = b - 1, m = (1 << bc) - 1;
+  if (T >= int64_t(1) << (3 * bc)) return;
+  fc[T] = mg_block_residual(1 << b, inv_dx2, f, p, int(T) & m, int(T >> bc) & m, int(T >> (2 * bc)));
   ec[T] = 0.0;
 }
 
-// phi += trilinear prolongation of the coarse correction
-__global__ void k_mg_prolong(int n, const double *__restrict__ ec, double *__restrict__ p) {
-  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (t >= int64_t(n) * n * n) return;
+// phi += trilinear prolongation of the coarse correction: the eight fine cells
+// of coarse cell (X, Y, Z), one axis after the other (3 a + b per axis, the
+// weights over 64; 46 FMAs for eight cells, against 12 operations per cell when
+// each forms its own weighted sum)
+__device__ __forceinline__ void mg_block_prolong(int n, const double *__restrict__ ec, double *__restrict__ p, int X,
+                                                 int Y, int Z) {
   const int h = n >> 1;
-  const int x = int(t % n), y = int((t / n) % n), z = int(t / (int64_t(n) * n));
-  const int X = x >> 1, Y = y >> 1, Z = z >> 1;
-  const int sx = (x & 1) ? 1 : -1, sy = (y & 1) ? 1 : -1, sz = (z & 1) ? 1 : -1;
-  double v = 27.0 * ec[mg_at(h, X, Y, Z)];
-  v += 9.0 * ((ec[mg_at(h, X + sx, Y, Z)] + ec[mg_at(h, X, Y + sy, Z)]) + ec[mg_at(h, X, Y, Z + sz)]);
-  v += 3.0 * ((ec[mg_at(h, X + sx, Y + sy, Z)] + ec[mg_at(h, X + sx, Y, Z + sz)]) +
-              ec[mg_at(h, X, Y + sy, Z + sz)]);
-  v += ec[mg_at(h, X + sx, Y + sy, Z + sz)];
-  p[t] += v / 64.0;
+  double zlo[2][2], zhi[2][2];  // [y][x] sums over z for the lower and the upper fine cells
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    double a[3][2];  // [j][x]
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const double c0 = ec[mg_at(h, X - 1, Y + j - 1, Z + k - 1)], c1 = ec[mg_at(h, X, Y + j - 1, Z + k - 1)],
+                   c2 = ec[mg_at(h, X + 1, Y + j - 1, Z + k - 1)];
+      a[j][0] = fma(3.0, c1, c0);
+      a[j][1] = fma(3.0, c1, c2);
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const double v[2] = {fma(3.0, a[1][x], a[0][x]), fma(3.0, a[1][x], a[2][x])};
+#pragma unroll
+      for (int y = 0; y < 2; ++y) {
+        if (k == 0) {
+          zlo[y][x] = v[y];
+        } else if (k == 1) {
+          zlo[y][x] = fma(3.0, v[y], zlo[y][x]);
+          zhi[y][x] = v[y];
+        } else {
+          zhi[y][x] = fma(3.0, zhi[y][x], v[y]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int z = 0; z < 2; ++z)
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      const int64_t i = mg_at(n, 2 * X, 2 * Y + y, 2 * Z + z);
+      double2 *q = reinterpret_cast<double2 *>(p + i);
+      double2 w = *q;
+      w.x = fma(z ? zhi[y][0] : zlo[y][0], 1.0 / 64.0, w.x);
+      w.y = fma(z ? zhi[y][1] : zlo[y][1], 1.0 / 64.0, w.y);
+      *q = w;
+    }
+}
+__global__ void k_mg_prolong(int b, const double *__restrict__ ec, double *__restrict__ p) {
+  const int64_t T = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  const int bc = b - 1, m = (1 << bc) - 1;
+  if (T >= int64_t(1) << (3 * bc)) return;
+  mg_block_prolong(1 << b, ec, p, int(T) & m, int(T >> bc) & m, int(T >> (2 * bc)));
 }
 
-// the 2^3 grid: `sweeps` red-black sweeps by one block of 8 threads
-__global__ void k_mg_coarsest(double dx2, const double *__restrict__ f, double *p, int sweeps) {
-  const int t = threadIdx.x;  // 0..7: (x, y, z) = bits of t
-  const int x = t & 1, y = (t >> 1) & 1, z = (t >> 2) & 1;
-  for (int s = 0; s < sweeps; ++s)
-    for (int colour = 0; colour < 2; ++colour) {
-      if (((x + y + z) & 1) == colour) {
-        const int64_t i = mg_at(2, x, y, z);
-        p[i] = (mg_nbsum(2, p, x, y, z) - dx2 * f[i]) * (1.0 / 6.0);
+// The rest of a V-cycle from a grid of n = 2^b <= 8 cells per axis down to 2^3
+// and back, by one block in shared memory (21 launches otherwise; a 16^3 grid's
+// FP64 work on one SM takes longer than its launches).
+constexpr int kMGTail = 8;
+__global__ void __launch_bounds__(256) k_mg_tail(int b, double dx2, const double *__restrict__ f, double *p, int pre,
+                                                 int post, int sweeps) {
+  __shared__ __align__(16) double sf[584], sp[584];  // 8^3 + 4^3 + 2^3
+  const int n3 = 1 << (3 * b);
+  for (int t = threadIdx.x; t < n3; t += blockDim.x) {
+    sf[t] = f[t];
+    sp[t] = p[t];
+  }
+  __syncthreads();
+  auto smooth = [&](int bb, int off, double d2, int ns) {
+    const int n = 1 << bb;
+    for (int s = 0; s < 2 * ns; ++s) {
+      for (int t = threadIdx.x; t < n * n * n / 2; t += blockDim.x) {
+        const int y = (t >> (bb - 1)) & (n - 1), z = t >> (2 * bb - 1);
+        const int x = 2 * (t & (n / 2 - 1)) + ((y + z + s) & 1);
+        const int64_t i = mg_at(n, x, y, z);
+        sp[off + i] = mg_sixth(mg_nbsum(n, sp + off, x, y, z) - d2 * sf[off + i]);
       }
       __syncthreads();
     }
+  };
+  int off = 0, bb = b;
+  double d2 = dx2;
+  while (bb > 1) {  // down
+    smooth(bb, off, d2, pre);
+    const int n = 1 << bb, nc = n / 2, offc = off + n * n * n;
+    for (int T = threadIdx.x; T < nc * nc * nc; T += blockDim.x) {
+      sf[offc + T] = mg_block_residual(n, 1.0 / d2, sf + off, sp + off, T & (nc - 1), (T >> (bb - 1)) & (nc - 1),
+                                       T >> (2 * bb - 2));
+      sp[offc + T] = 0.0;
+    }
+    __syncthreads();
+    off = offc;
+    --bb;
+    d2 *= 4.0;
+  }
+  smooth(bb, off, d2, sweeps);
+  while (bb < b) {  // up
+    ++bb;
+    const int n = 1 << bb, nc = n / 2, offc = off;
+    off -= n * n * n;
+    d2 *= 0.25;
+    for (int T = threadIdx.x; T < nc * nc * nc; T += blockDim.x)
+      mg_block_prolong(n, sp + offc, sp + off, T & (nc - 1), (T >> (bb - 1)) & (nc - 1), T >> (2 * bb - 2));
+    __syncthreads();
+    smooth(bb, off, d2, post);
+  }
+  for (int t = threadIdx.x; t < n3; t += blockDim.x) p[t] = sp[t];
 }
 
 // residual of the base level into r (for its L2 norm)
@@ -156,10 +257,8 @@ __global__ void k_mg_residual(int n, double inv_dx2, const double *__restrict__ 
 
 // sqrt of the sum of the partial sums into out
 __global__ void k_mg_norm(const double *__restrict__ part, int nparts, double *__restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0.0;
-  for (int q = 0; q < nparts; ++q) s += part[q];
-  *out = sqrt(s);
+  const double s = mg_sum_parts(part, nparts);
+  if (threadIdx.x == 0) *out = sqrt(s);
 }
 
 // phi - mean into the octs' cells (mesh order)
@@ -179,9 +278,10 @@ __global__ void k_mg_scatter(const double *__restrict__ p, const uint64_t *__res
 // Poisson on a refined level (Sec. 5, level by level): flat tables over the
 // cells of each MG level (level 0: the level's cells; level k: their
 // ancestors at level L-k), built on the host once per (member, level).
-// Every operation is rounded as written (no contraction), in the order of the
-// plain definition, so the potential equals that of a sequential evaluation
-// bit for bit.
+// Every operation is rounded as written (no contraction; a division by a power
+// of two is the exact product with its reciprocal, one by 6..12 see
+// mgl_over_diag), in the order of the plain definition, so the potential equals
+// that of a sequential evaluation bit for bit.
 //   nb[6][n]   face neighbour in the same MG level (-x,+x,-y,+y,-z,+z) or -1
 //   nbnd[n]    faces to the outside (Dirichlet): the diagonal is -(6 + nbnd)
 //   bsum[n]    2 sum of the faces' boundary values (MG level 0; 0 above)
@@ -225,6 +325,19 @@ __global__ void k_mgl_scatter(int64_t n, const int32_t *__restrict__ g0, const d
   if (t < n) phil[g0[t]] = e[t];
 }
 
+// x / (6 + b) rounded to nearest for b in 0..6, without a division: with y the
+// rounded reciprocal (|1 - d y| is at most 2^-54 for these divisors), q = x y is
+// within an ulp of the quotient and one step q + y (x - d q) rounds correctly
+// (Markstein, IBM J. Res. Dev. 34, 1990).  Outside the range where the residual
+// is exact (tiny, huge or non-finite x) the division itself.
+__constant__ double kDiag[7] = {6.0, 7.0, 8.0, 9.0, 10.0, 11.0, 12.0};
+__constant__ double kRcpDiag[7] = {1.0 / 6.0, 1.0 / 7.0, 1.0 / 8.0, 1.0 / 9.0, 1.0 / 10.0, 1.0 / 11.0, 1.0 / 12.0};
+__device__ __forceinline__ double mgl_over_diag(double x, int b) {
+  if (!within<900>(fabs(x))) return __ddiv_rn(x, kDiag[b]);
+  const double d = kDiag[b], y = kRcpDiag[b], q = mul_int(x, y);
+  return __fma_rn(y, __fma_rn(-d, q, x), q);
+}
+
 __device__ __forceinline__ double mgl_nbsum(int64_t n, const int32_t *__restrict__ nb, const double *e, int64_t t) {
   double s = 0.0;
 #pragma unroll
@@ -244,17 +357,36 @@ __global__ void k_mgl_smooth(int64_t n, const int32_t *__restrict__ list, int64_
   const int64_t t = list[i];
   const double s = mgl_nbsum(n, nb, e, t);
   const double bs = bsum ? bsum[t] : 0.0;
-  e[t] = __ddiv_rn(__dsub_rn(__dadd_rn(s, bs), __dmul_rn(dx2, f[t])), double(6 + nbnd[t]));
+  e[t] = mgl_over_diag(__dsub_rn(__dadd_rn(s, bs), __dmul_rn(dx2, f[t])), nbnd[t]);
+}
+
+// `sweeps` red-black sweeps of a small MG level (its even cells first in list)
+// by one block: a launch per colour costs more than its few cells
+constexpr int64_t kMGLBlock = 1024;
+__global__ void __launch_bounds__(512) k_mgl_sweeps(int64_t n, const int32_t *__restrict__ list, int64_t nc0,
+                                                    const int32_t *__restrict__ nb, const int32_t *__restrict__ nbnd,
+                                                    const double *__restrict__ bsum, const double *__restrict__ f,
+                                                    double *e, double dx2, int sweeps) {
+  for (int s = 0; s < 2 * sweeps; ++s) {
+    const int64_t i1 = (s & 1) ? n : nc0;
+    for (int64_t i = ((s & 1) ? nc0 : 0) + threadIdx.x; i < i1; i += blockDim.x) {
+      const int64_t t = list[i];
+      const double sum = mgl_nbsum(n, nb, e, t);
+      const double bs = bsum ? bsum[t] : 0.0;
+      e[t] = mgl_over_diag(__dsub_rn(__dadd_rn(sum, bs), __dmul_rn(dx2, f[t])), nbnd[t]);
+    }
+    __syncthreads();
+  }
 }
 
 __global__ void k_mgl_residual(int64_t n, const int32_t *__restrict__ nb, const int32_t *__restrict__ nbnd,
                                const double *__restrict__ bsum, const double *__restrict__ f,
-                               const double *__restrict__ e, double dx2, double *__restrict__ r) {
+                               const double *__restrict__ e, double inv_dx2, double *__restrict__ r) {
   const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (t >= n) return;
   const double s = mgl_nbsum(n, nb, e, t);
   const double bs = bsum ? bsum[t] : 0.0;
-  r[t] = __dsub_rn(f[t], __ddiv_rn(__dsub_rn(__dadd_rn(s, bs), __dmul_rn(double(6 + nbnd[t]), e[t])), dx2));
+  r[t] = __dsub_rn(f[t], __dmul_rn(__dsub_rn(__dadd_rn(s, bs), __dmul_rn(kDiag[nbnd[t]], e[t])), inv_dx2));
 }
 
 // coarse source = the children's residuals summed over 8; correction zeroed
@@ -268,7 +400,7 @@ __global__ void k_mgl_restrict(int64_t nc, const int32_t *__restrict__ child, co
     const int32_t q = child[j * nc + t];
     if (q >= 0) s = __dadd_rn(s, r[q]);
   }
-  fc[t] = __ddiv_rn(s, 8.0);
+  fc[t] = __dmul_rn(s, 0.125);
   ec[t] = 0.0;
 }
 
@@ -287,7 +419,7 @@ __global__ void k_mgl_prolong(int64_t nf, const int32_t *__restrict__ pro, const
   v = __dadd_rn(v, __dmul_rn(9.0, __dadd_rn(__dadd_rn(c[4], c[2]), c[1])));
   v = __dadd_rn(v, __dmul_rn(3.0, __dadd_rn(__dadd_rn(c[6], c[5]), c[3])));
   v = __dadd_rn(v, c[7]);
-  e[t] = __dadd_rn(e[t], __ddiv_rn(v, 64.0));
+  e[t] = __dadd_rn(e[t], __dmul_rn(v, 1.0 / 64.0));
 }
 
 // sum of r^2 into one value per block (for the residual norm)
@@ -308,10 +440,8 @@ __global__ void k_mgl_sq(int64_t n, const double *__restrict__ r, double *__rest
 }
 
 __global__ void k_mgl_norm(const double *__restrict__ part, int nparts, double *out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0.0;
-  for (int b = 0; b < nparts; ++b) s += part[b];
-  *out = sqrt(s);
+  const double s = mg_sum_parts(part, nparts);
+  if (threadIdx.x == 0) *out = sqrt(s);
 }
 
 // ---------------------------------------------------------------------------
