@@ -802,14 +802,15 @@ static StepArgs<T> step_args(amr_mesh *h, bool device_dt, double dt) {
   return a;
 }
 
-// persistent grid: enough blocks to fill the GPU once, never more than tiles;
-// smem: bytes of dynamic shared memory per thread
+// persistent grid: enough blocks to fill the GPU once, never more than tiles.
+// smem: bytes of dynamic shared memory per thread; per_tile: blocks that share a
+// tile (3: one per axis)
 template <class T>
 static void run_list(amr_mesh *h, int kid, void (*kern)(StepArgs<T>), StepArgs<T> a,
-                     const SegList &L, int dom, size_t smem = 0) {
+                     const SegList &L, int dom, size_t smem = 0, int per_tile = 1) {
   if (L.ntile[dom] == 0) return;
   a.tiles = tile_list(h, L, dom);
-  int grid = a.tiles.ntiles;
+  int grid = a.tiles.ntiles * per_tile;
   if (h->persistent) {
     int per_sm = 0;
     for (auto &o : h->occ)
@@ -823,7 +824,7 @@ static void run_list(amr_mesh *h, int kid, void (*kern)(StepArgs<T>), StepArgs<T
       }
       h->occ.push_back({(const void *)kern, per_sm});
     }
-    grid = std::min(a.tiles.ntiles, per_sm * h->sm_count);
+    grid = std::min(grid, per_sm * h->sm_count);
   }
   launch_smem(h, kid, kern, dim3(unsigned(grid)), dim3(unsigned(h->tile_size)), smem * h->tile_size, a);
 }
@@ -917,14 +918,14 @@ static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double d
   } else if constexpr (sizeof(T) == 4) {
     // FP32: primitives recomputed inside the predictor; each leaf cell solves
     // its six faces and updates itself
-    run_list(h, K_PREDICT, k_predict_u<T>, a, L, DOM_CELLS);
+    run_list(h, K_PREDICT, k_predict_u, a, L, DOM_CELLS);
     run_list(h, K_FLUX, k_flux_update, a, L, DOM_REAL, 20);
     if (L.ntile[DOM_REFLUX]) *pend = &L;
   } else {
     // FP64: every predictor and every face solve exactly once
     run_list(h, K_PRIM, k_ghost_prim, a, L, DOM_CELLS, 16);
     run_list(h, K_PREDICT, k_predict, a, L, DOM_CELLS);
-    run_list(h, K_FLUX, k_flux<T>, a, L, DOM_CELLS);
+    run_list(h, K_FLUX, k_flux, a, L, DOM_CELLS, 0, 3);
     run_list(h, K_UPDATE, k_update, a, L, DOM_UPDATE, 40);
   }
 }
