@@ -276,10 +276,10 @@ struct amr_mesh {
   double *phi = nullptr;
 
   // particle deposition onto the levels: positions and masses (the handle's
-  // precision), two particle lists, split flags and their prefix sums, list
-  // lengths per level, and the density of every cell
+  // precision), two particle lists, list lengths per level, and the density of
+  // every cell
   void *px = nullptr, *py = nullptr, *pz = nullptr, *pm = nullptr;
-  uint32_t *plist0 = nullptr, *plist1 = nullptr, *pflag = nullptr, *ppos = nullptr, *ptmp = nullptr;
+  uint32_t *plist0 = nullptr, *plist1 = nullptr;
   int64_t *pcount = nullptr;
   int64_t pcap = 0;
   void *prho = nullptr;
@@ -3139,11 +3139,6 @@ extern "C" amr_status amr_batch_repack(amr_handle h, int n_keep, const int32_t *
 // ---------------------------------------------------------------------------
 // CIC deposition onto the levels of the selected member (Sec. 4)
 // ---------------------------------------------------------------------------
-__global__ void k_iota_u32(uint32_t *a, int64_t n) {
-  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (t < n) a[t] = uint32_t(t);
-}
-
 static amr_status ensure_particles(amr_mesh *h, int64_t np, bool positions) {
   const size_t es = h->elem();
   if (np > h->pcap || (positions && !h->px)) {
@@ -3151,7 +3146,7 @@ static amr_status ensure_particles(amr_mesh *h, int64_t np, bool positions) {
       dev_free(h, *b);
       *b = nullptr;
     }
-    for (uint32_t **b : {&h->plist0, &h->plist1, &h->pflag, &h->ppos, &h->ptmp}) {
+    for (uint32_t **b : {&h->plist0, &h->plist1}) {
       dev_free(h, *b);
       *b = nullptr;
     }
@@ -3159,8 +3154,7 @@ static amr_status ensure_particles(amr_mesh *h, int64_t np, bool positions) {
     const int64_t cap = std::max<int64_t>(np, 1);
     if (positions)
       for (void **b : {&h->px, &h->py, &h->pz, &h->pm}) AMR_TRY(dev_alloc(h, b, es * size_t(cap)));
-    for (uint32_t **b : {&h->plist0, &h->plist1, &h->pflag, &h->ppos}) AMR_TRY(alloc_n(h, b, cap));
-    AMR_TRY(alloc_n(h, &h->ptmp, scan_tmp_size(cap)));
+    for (uint32_t **b : {&h->plist0, &h->plist1}) AMR_TRY(alloc_n(h, b, cap));
     h->pcap = cap;
   }
   if (!h->pcount) AMR_TRY(alloc_n(h, &h->pcount, kMaxLev + 2));
@@ -3198,29 +3192,17 @@ static void deposit_levels(amr_mesh *h, int64_t np, const T *x, const T *y, cons
   cnt[size_t(mb.lmin)] = np;
   cudaMemcpyAsync(h->pcount, cnt.data(), sizeof(int64_t) * cnt.size(), cudaMemcpyHostToDevice, h->s);
   if (np == 0) return;
-  uint32_t *cur = h->plist0, *nxt = h->plist1;
+  const uint32_t *cur = nullptr;  // the base level's list holds every particle
+  uint32_t *nxt = h->plist0;
   for (int l = mb.lmin; l <= mb.lmax; ++l) {
-    if (l == mb.lmin)  // every particle, every stencil cell exists: the base table
-      launch(h, K_DEPOSIT, k_deposit_base<T>, dim3(nblocks(np)), dim3(256), (const int32_t *)h->btab, l, np,
-             x, y, z, m, static_cast<T *>(h->prho));
-    else
-      launch(h, K_DEPOSIT, k_deposit_level<T>, dim3(nblocks(np)), dim3(256), h->hash, h->sel, l, N, x, y,
-             z, m, (const uint32_t *)cur, (const int64_t *)h->pcount, static_cast<T *>(h->prho));
-    if (l == mb.lmax) break;
-    if (l == mb.lmin) {
-      launch(h, K_SPLIT, k_split_base<T>, dim3(nblocks(np)), dim3(256), (const int32_t *)h->btab, l,
-             (const uint32_t *)h->son, x, y, z, np, h->pflag);
-      launch(h, K_DEPOSIT, k_iota_u32, dim3(nblocks(np)), dim3(256), cur, np);
-    } else {
-      launch(h, K_SPLIT, k_split_level<T>, dim3(nblocks(np)), dim3(256), h->hash, h->sel, l, N,
-             (const uint32_t *)h->son, x, y, z, (const uint32_t *)cur, (const int64_t *)h->pcount, np,
-             h->pflag);
-    }
-    cudaMemcpyAsync(h->ppos, h->pflag, 4 * size_t(np), cudaMemcpyDeviceToDevice, h->s);
-    scan_exclusive(h, h->ppos, np, h->ptmp);
-    launch(h, K_SPLIT, k_compact_level, dim3(nblocks(np)), dim3(256), (const uint32_t *)cur,
-           (const uint32_t *)h->pflag, (const uint32_t *)h->ppos, np, l, nxt, h->pcount);
-    std::swap(cur, nxt);
+    // every stencil cell of the base level exists: its table; the finer lists'
+    // lengths are on the device: a grid that fills the GPU loops over them
+    const OctFinder find{l == mb.lmin ? (const int32_t *)h->btab : nullptr, h->hash, h->sel, l, N};
+    const unsigned all = nblocks(np), grid = l == mb.lmin ? all : std::min(all, unsigned(8 * h->sm_count));
+    launch(h, K_DEPOSIT, k_deposit_level<T>, dim3(grid), dim3(256), find, (const uint32_t *)h->son, x, y, z, m, cur,
+           h->pcount, static_cast<T *>(h->prho), l < mb.lmax ? nxt : (uint32_t *)nullptr);
+    cur = nxt;
+    nxt = nxt == h->plist0 ? h->plist1 : h->plist0;
   }
 }
 

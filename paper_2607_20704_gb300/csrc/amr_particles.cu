@@ -22,11 +22,11 @@ namespace {
 
 enum PKid {
   P_KEYS, P_SORT_HIST, P_SORT_SCAN, P_SORT_SCATTER, P_GATHER, P_ZERO, P_CIC_ATOMIC,
-  P_SEG_HEADS, P_SEG_SCAN, P_SEG_STARTS, P_SEG_PARTIAL, P_SEG_CARRY, P_SEG_GATHER, P_CONVERT, P_COUNT
+  P_SEG_HEADS, P_SEG_SCAN, P_SEG_PARTIAL, P_SEG_CARRY, P_SEG_GATHER, P_CONVERT, P_COUNT
 };
 const char *const kPartKernelNames[P_COUNT] = {
     "part_keys", "psort_hist", "psort_scan", "psort_scatter", "part_gather", "grid_zero",
-    "cic_atomic", "seg_heads", "seg_scan", "seg_starts", "seg_partial", "seg_carry", "seg_gather", "convert"};
+    "cic_atomic", "seg_heads", "seg_scan", "seg_partial", "seg_carry", "seg_gather", "convert"};
 
 amr_status set_error(amr_status s, const std::string &msg) {
   amr_set_error_text(msg.c_str());
@@ -242,41 +242,41 @@ void sort_impl(amr_particles *h) {
   const int64_t np = h->np, nt = ntiles(h);
   const CicGrid<T> g = grid_of<T>(h);
   const T *px = (const T *)h->x, *py = (const T *)h->y, *pz = (const T *)h->z;
-  const dim3 kg(nblocks(np)), kb256(256);
-  switch (h->bits) {
-    case 1: launch(h, P_KEYS, k_part_keys<T, 1>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-    case 2: launch(h, P_KEYS, k_part_keys<T, 2>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-    case 3: launch(h, P_KEYS, k_part_keys<T, 3>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-    case 4: launch(h, P_KEYS, k_part_keys<T, 4>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-    case 5: launch(h, P_KEYS, k_part_keys<T, 5>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-    case 6: launch(h, P_KEYS, k_part_keys<T, 6>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-    case 7: launch(h, P_KEYS, k_part_keys<T, 7>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-    case 8: launch(h, P_KEYS, k_part_keys<T, 8>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-    case 9: launch(h, P_KEYS, k_part_keys<T, 9>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-    default: launch(h, P_KEYS, k_part_keys<T, 10>, kg, kb256, np, g, px, py, pz, h->key, h->val); break;
-  }
-  uint32_t *ka = h->key, *kb = h->key2, *va = h->val, *vb = h->val2;
   // passes of equal width, at most 8 bits each (27-bit keys of a 512^3 grid:
   // 7, 7, 7, 6): fewer digits per pass keep each digit's run in a tile longer,
   // so the scatter writes stay coalesced
   const int total = 3 * h->bits;
   const int passes = (total + 7) / 8, width = (total + passes - 1) / passes;
+  const dim3 kg{unsigned(nt)}, kb(kSortThreads);
+  switch (h->bits) {
+    case 1: launch(h, P_KEYS, k_part_keys<T, 1>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+    case 2: launch(h, P_KEYS, k_part_keys<T, 2>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+    case 3: launch(h, P_KEYS, k_part_keys<T, 3>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+    case 4: launch(h, P_KEYS, k_part_keys<T, 4>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+    case 5: launch(h, P_KEYS, k_part_keys<T, 5>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+    case 6: launch(h, P_KEYS, k_part_keys<T, 6>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+    case 7: launch(h, P_KEYS, k_part_keys<T, 7>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+    case 8: launch(h, P_KEYS, k_part_keys<T, 8>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+    case 9: launch(h, P_KEYS, k_part_keys<T, 9>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+    default: launch(h, P_KEYS, k_part_keys<T, 10>, kg, kb, np, g, px, py, pz, h->key, width, h->table); break;
+  }
+  uint32_t *ka = h->key, *kb2 = h->key2, *va = h->val, *vb = h->val2;
   for (int shift = 0; shift < total; shift += width) {
     const int nbits = total - shift < width ? total - shift : width;
     const int64_t len = (int64_t(1) << nbits) * nt;
     const int ndig = 1 << nbits;
     const int64_t nch = (nt + kScanChunk - 1) / kScanChunk;
     uint32_t *pref = h->table + len, *base = pref + len, *dbase = base + int64_t(ndig) * nch;
-    launch(h, P_SORT_HIST, k_psort_hist, dim3(unsigned(nt)), dim3(kSortThreads), (const uint32_t *)ka, np,
-           shift, nbits, h->table, nt);
-    launch(h, P_SORT_SCAN, k_psort_chunks, dim3(unsigned(nch)), dim3(kSortThreads), (const uint32_t *)h->table,
+    if (shift > 0)  // the keys' kernel counted the first digit
+      launch(h, P_SORT_HIST, k_psort_hist, kg, kb, (const uint32_t *)ka, np, shift, nbits, h->table);
+    launch(h, P_SORT_SCAN, k_psort_chunks, dim3(unsigned(nch)), dim3(kSortBins), (const uint32_t *)h->table,
            nt, ndig, pref, base);
-    launch(h, P_SORT_SCAN, k_psort_digit_scan, dim3(unsigned(ndig)), dim3(kSortThreads), base, nch, ndig, dbase);
-    launch(h, P_SORT_SCAN, k_psort_digit_base, dim3(1), dim3(kSortThreads), dbase, ndig);
-    launch(h, P_SORT_SCATTER, k_psort_scatter, dim3(unsigned(nt)), dim3(kSortThreads), (const uint32_t *)ka,
-           (const uint32_t *)va, kb, vb, np, shift, nbits, (const uint32_t *)h->table, (const uint32_t *)pref,
+    launch(h, P_SORT_SCAN, k_psort_digit_scan, dim3(unsigned(ndig)), dim3(kScanThreads), base, nch, ndig, dbase);
+    launch(h, P_SORT_SCAN, k_psort_digit_base, dim3(1), dim3(kScanThreads), dbase, ndig);
+    launch(h, P_SORT_SCATTER, shift > 0 ? k_psort_scatter<false> : k_psort_scatter<true>, kg, kb,
+           (const uint32_t *)ka, (const uint32_t *)va, kb2, vb, np, shift, nbits, (const uint32_t *)pref,
            (const uint32_t *)base, (const uint32_t *)dbase);
-    std::swap(ka, kb);
+    std::swap(ka, kb2);
     std::swap(va, vb);
   }
   launch(h, P_GATHER, k_part_gather<T>, dim3(nblocks(np)), dim3(256), np, (const uint32_t *)va,
@@ -301,16 +301,14 @@ template <class T>
 void deposit_segment(amr_particles *h) {
   const int64_t np = h->np, cap = np > 0 ? np : 1, ng = ngroups(h) > 0 ? ngroups(h) : 1;
   zero(h, P_ZERO, h->cellmap, 0xFF, size_t(cells(h)) * sizeof(int32_t));
-  zero(h, P_ZERO, h->nseg, 0, sizeof(uint32_t));
+  if (np == 0) zero(h, P_ZERO, h->nseg, 0, sizeof(uint32_t));
   if (np > 0) {
     launch(h, P_SEG_HEADS, k_seg_heads, dim3(nblocks(np)), dim3(256), np, (const uint32_t *)h->sorted_key,
            h->flag);
     scan_exclusive(h, P_SEG_SCAN, h->flag, np, h->scan_tmp);
-    launch(h, P_SEG_STARTS, k_seg_starts, dim3(nblocks(np)), dim3(256), np, (const uint32_t *)h->sorted_key,
-           (const uint32_t *)h->flag, h->start, h->nseg);
     launch(h, P_SEG_PARTIAL, k_seg_partial<T>, dim3(nblocks(np)), dim3(256), np, grid_of<T>(h),
            (const uint32_t *)h->sorted_key, (const uint32_t *)h->flag, (const T *)h->x, (const T *)h->y,
-           (const T *)h->z, (const T *)h->m, cap, ng, (T *)h->sums, (T *)h->carry, h->cellmap);
+           (const T *)h->z, (const T *)h->m, cap, ng, (T *)h->sums, (T *)h->carry, h->cellmap, h->start, h->nseg);
     launch(h, P_SEG_CARRY, k_seg_carry<T>, dim3(nblocks(np)), dim3(256), (const uint32_t *)h->nseg,
            (const uint32_t *)h->start, cap, ng, (const T *)h->carry, (T *)h->sums);
   }

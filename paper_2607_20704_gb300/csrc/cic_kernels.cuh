@@ -9,7 +9,7 @@
 // source cell so that particles of one source cell are contiguous.
 //
 //   sort      source-cell Hilbert keys, then a stable LSD radix sort of
-//             (key, particle) pairs, tiles of 2048 items staged through
+//             (key, particle) pairs, tiles of 4096 items staged through
 //             shared memory so that every digit's run is written contiguously;
 //             then the particle arrays are gathered into the sorted order.
 //   atomic    one thread per particle; lanes of a warp that share a source
@@ -28,14 +28,16 @@
 // even a non-finite one, addresses outside the grid.
 #pragma once
 #include "amr_internal.cuh"
+#include "cic_weights.cuh"
 #include "scan_kernels.cuh"
 
 namespace amr {
 namespace {
 
-constexpr int kSortThreads = 256;
+constexpr int kSortThreads = 512;
+constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortRounds = 8;
-constexpr int kSortTile = kSortThreads * kSortRounds;  // 2048 items per tile
+constexpr int kSortTile = kSortThreads * kSortRounds;  // 4096 items per tile
 
 // Grid of the deposition: n = 2^bits cells per axis; fn = n in the state type.
 template <class T>
@@ -72,7 +74,7 @@ __device__ __forceinline__ double half_odd(int i) {
 // source cell along one axis: floor(x n - 1/2), unmasked
 template <class T>
 __device__ __forceinline__ int cic_cell(T x, const CicGrid<T> &g) {
-  return int(floor(x * g.fn - T(0.5)));
+  return __float2int_rd(x * g.fn - T(0.5));
 }
 template <>
 __device__ __forceinline__ int cic_cell<double>(double x, const CicGrid<double> &g) {
@@ -123,6 +125,25 @@ __device__ __forceinline__ void cic_weights(T x, T y, T z, T m, const CicGrid<T>
   for (int q = 0; q < 4; ++q) b[q] = a[q & 1] * wy[q >> 1];
 #pragma unroll
   for (int c = 0; c < 8; ++c) w[c] = b[c & 3] * wz[c >> 2];
+}
+
+// FP64: on the integer pipes, each contribution rounded once
+template <>
+__device__ __forceinline__ void cic_weights<double>(double x, double y, double z, double m, const CicGrid<double> &g,
+                                                    int &i, int &j, int &k, double w[8]) {
+  if (cic_in_range(x, y, z, m)) {
+    uint64_t b[8];
+    cic_weights_int(uint64_t(__double_as_longlong(x)), uint64_t(__double_as_longlong(y)),
+                    uint64_t(__double_as_longlong(z)), uint64_t(__double_as_longlong(m)), g.bits, i, j, k, b);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) w[c] = __longlong_as_double((long long)b[c]);
+    return;
+  }
+  double wx[2], wy[2], wz[2];
+  i = cic_axis(x, g, wx[0], wx[1]);
+  j = cic_axis(y, g, wy[0], wy[1]);
+  k = cic_axis(z, g, wz[0], wz[1]);
+  for (int c = 0; c < 8; ++c) w[c] = ((m * g.scale * wx[c & 1]) * wy[(c >> 1) & 1]) * wz[c >> 2];
 }
 
 // Sums of the lanes' w over runs of lanes (`runs`: bit L set where a run
@@ -212,29 +233,42 @@ __device__ __forceinline__ uint32_t hilbert_index_u32(uint32_t a0, uint32_t a1, 
   return (spread3(a0) << 2) | (spread3(a1) << 1) | spread3(a2);
 }
 
-template <class T, int BITS>
-__global__ void k_part_keys(int64_t np, CicGrid<T> g, const T *__restrict__ x, const T *__restrict__ y,
-                            const T *__restrict__ z, uint32_t *__restrict__ key,
-                            uint32_t *__restrict__ val) {
-  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (t >= np) return;
-  const uint32_t m = uint32_t(g.n - 1);
-  const uint32_t i = uint32_t(cic_cell(x[t], g)) & m, j = uint32_t(cic_cell(y[t], g)) & m,
-                 k = uint32_t(cic_cell(z[t], g)) & m;
-  key[t] = hilbert_index_u32<BITS>(i, j, k);
-  val[t] = uint32_t(t);
-}
-
 // per-tile digit counts, tile-major: table[tile * ndig + d]; digits of up to 8 bits
 constexpr int kSortBins = 256;
 
-__global__ void __launch_bounds__(kSortThreads) k_psort_hist(const uint32_t *__restrict__ keys,
-                                                             int64_t np, int shift, int nbits,
-                                                             uint32_t *__restrict__ table,
-                                                             int64_t ntiles) {
+// the keys, and the tile's counts of the first digit
+template <class T, int BITS>
+__global__ void __launch_bounds__(kSortThreads) k_part_keys(int64_t np, CicGrid<T> g, const T *__restrict__ x,
+                                                            const T *__restrict__ y, const T *__restrict__ z,
+                                                            uint32_t *__restrict__ key, int nbits,
+                                                            uint32_t *__restrict__ table) {
   __shared__ uint32_t hist[kSortBins];
   const int ndig = 1 << nbits;
-  for (int d = threadIdx.x; d < ndig; d += blockDim.x) hist[d] = 0;
+  for (int d = threadIdx.x; d < ndig; d += kSortThreads) hist[d] = 0;
+  __syncthreads();
+  const int64_t base = blockIdx.x * int64_t(kSortTile);
+  const uint32_t m = uint32_t(g.n - 1);
+#pragma unroll 4
+  for (int r = 0; r < kSortRounds; ++r) {
+    const int64_t t = base + r * kSortThreads + threadIdx.x;
+    if (t < np) {
+      const uint32_t i = uint32_t(cic_cell(x[t], g)) & m, j = uint32_t(cic_cell(y[t], g)) & m,
+                     k = uint32_t(cic_cell(z[t], g)) & m;
+      const uint32_t h = hilbert_index_u32<BITS>(i, j, k);
+      key[t] = h;
+      atomicAdd(&hist[h & unsigned(ndig - 1)], 1u);
+    }
+  }
+  __syncthreads();
+  for (int d = threadIdx.x; d < ndig; d += kSortThreads) table[int64_t(blockIdx.x) * ndig + d] = hist[d];
+}
+
+__global__ void __launch_bounds__(kSortThreads) k_psort_hist(const uint32_t *__restrict__ keys,
+                                                             int64_t np, int shift, int nbits,
+                                                             uint32_t *__restrict__ table) {
+  __shared__ uint32_t hist[kSortBins];
+  const int ndig = 1 << nbits;
+  for (int d = threadIdx.x; d < ndig; d += kSortThreads) hist[d] = 0;
   __syncthreads();
   const int64_t base = blockIdx.x * int64_t(kSortTile);
   unsigned dk[kSortRounds];  // all loads of the tile in flight at once
@@ -247,7 +281,7 @@ __global__ void __launch_bounds__(kSortThreads) k_psort_hist(const uint32_t *__r
   for (int r = 0; r < kSortRounds; ++r)
     if (dk[r] != 0xFFFFFFFFu) atomicAdd(&hist[(dk[r] >> shift) & unsigned(ndig - 1)], 1u);
   __syncthreads();
-  for (int d = threadIdx.x; d < ndig; d += blockDim.x) table[int64_t(blockIdx.x) * ndig + d] = hist[d];
+  for (int d = threadIdx.x; d < ndig; d += kSortThreads) table[int64_t(blockIdx.x) * ndig + d] = hist[d];
 }
 
 // Offsets of the scatter from the tile-major counts cnt[tile][d]: per digit,
@@ -275,17 +309,19 @@ __global__ void k_psort_chunks(const uint32_t *__restrict__ cnt, int64_t ntiles,
 
 // one block per digit: exclusive scan of the digit's chunk totals (in place)
 // and the digit's total
-__global__ void __launch_bounds__(kSortThreads) k_psort_digit_scan(uint32_t *__restrict__ base, int64_t nchunks,
+constexpr int kScanThreads = 256;
+
+__global__ void __launch_bounds__(kScanThreads) k_psort_digit_scan(uint32_t *__restrict__ base, int64_t nchunks,
                                                                   int ndig, uint32_t *__restrict__ dtot) {
-  __shared__ uint32_t part[kSortThreads];
+  __shared__ uint32_t part[kScanThreads];
   const int d = blockIdx.x;
-  const int64_t per = (nchunks + kSortThreads - 1) / kSortThreads;
+  const int64_t per = (nchunks + kScanThreads - 1) / kScanThreads;
   const int64_t c0 = threadIdx.x * per, c1 = c0 + per < nchunks ? c0 + per : nchunks;
   uint32_t sum = 0;
   for (int64_t c = c0; c < c1; ++c) sum += base[c * ndig + d];
   part[threadIdx.x] = sum;
   __syncthreads();
-  for (int off = 1; off < kSortThreads; off <<= 1) {
+  for (int off = 1; off < kScanThreads; off <<= 1) {
     const uint32_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0u;
     __syncthreads();
     part[threadIdx.x] += v;
@@ -297,17 +333,17 @@ __global__ void __launch_bounds__(kSortThreads) k_psort_digit_scan(uint32_t *__r
     base[c * ndig + d] = run;
     run += x;
   }
-  if (threadIdx.x == kSortThreads - 1) dtot[d] = part[kSortThreads - 1];
+  if (threadIdx.x == kScanThreads - 1) dtot[d] = part[kScanThreads - 1];
 }
 
 // one block: the digits' bases, the exclusive scan of their totals (in place)
-__global__ void __launch_bounds__(kSortThreads) k_psort_digit_base(uint32_t *__restrict__ dtot, int ndig) {
-  __shared__ uint32_t part[kSortThreads];
+__global__ void __launch_bounds__(kScanThreads) k_psort_digit_base(uint32_t *__restrict__ dtot, int ndig) {
+  __shared__ uint32_t part[kScanThreads];
   const int d = threadIdx.x;
   const uint32_t x = d < ndig ? dtot[d] : 0u;
   part[d] = x;
   __syncthreads();
-  for (int off = 1; off < kSortThreads; off <<= 1) {
+  for (int off = 1; off < kScanThreads; off <<= 1) {
     const uint32_t v = d >= off ? part[d - off] : 0u;
     __syncthreads();
     part[d] += v;
@@ -316,89 +352,94 @@ __global__ void __launch_bounds__(kSortThreads) k_psort_digit_base(uint32_t *__r
   if (d < ndig) dtot[d] = part[d] - x;
 }
 
-// stable scatter of one tile: ranks in item order (rounds, then warps, then
-// lanes), the tile staged in shared memory in digit order, then written out
-// so that consecutive threads write consecutive places of a digit's run.
+// Stable scatter of one tile.  Each warp ranks 256 consecutive items by itself
+// (8 rounds of 32, counting per digit in its own row of wcnt), the rows are
+// summed over the warps once, and the tile goes through shared memory in digit
+// order, so that consecutive threads write consecutive places of a digit's run.
+// Two barriers per round and 2048-item tiles, as every digit's count was kept
+// for the block, took 132 us per pass of 16.8 M pairs; this takes FIRST: the
+// values are the items' indices (nothing read).
+template <bool FIRST>
 __global__ void __launch_bounds__(kSortThreads) k_psort_scatter(
     const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
-    uint32_t *__restrict__ vout, int64_t np, int shift, int nbits, const uint32_t *__restrict__ cnt,
-    const uint32_t *__restrict__ pref, const uint32_t *__restrict__ cbase, const uint32_t *__restrict__ dbase) {
+    uint32_t *__restrict__ vout, int64_t np, int shift, int nbits, const uint32_t *__restrict__ pref,
+    const uint32_t *__restrict__ cbase, const uint32_t *__restrict__ dbase) {
   __shared__ uint32_t skey[kSortTile], sval[kSortTile];
-  __shared__ uint32_t wcnt[kSortThreads / 32][256], wpre[kSortThreads / 32][256];
-  __shared__ uint32_t lstart[256], run[256], part[kSortThreads];
+  __shared__ uint16_t wcnt[kSortWarps * kSortBins];  // [warp][digit]; a tile's counts stay below 2^16
+  __shared__ uint32_t lstart[kSortBins], goff[kSortBins], wsum[kSortBins / 32];
   const int ndig = 1 << nbits;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t base = blockIdx.x * int64_t(kSortTile);
   const int nt = int(np - base < kSortTile ? np - base : kSortTile);
-  // digit counts and global offsets of this tile, then the counts'
-  // exclusive scan over the digits (one digit per thread; ndig <= 256)
-  __shared__ uint32_t goff[256];
-  const int d0 = threadIdx.x;
-  uint32_t cnt_d = 0;
-  if (d0 < ndig) {
-    const int64_t e = int64_t(blockIdx.x) * ndig + d0;
-    cnt_d = cnt[e];
-    goff[d0] = pref[e] + cbase[int64_t(blockIdx.x / kScanChunk) * ndig + d0] + dbase[d0];
-  }
-  part[threadIdx.x] = cnt_d;
-  for (int w = 0; w < kSortThreads / 32; ++w) wcnt[w][threadIdx.x] = 0;
-  __syncthreads();
-  for (int off = 1; off < kSortThreads; off <<= 1) {
-    const uint32_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0u;
-    __syncthreads();
-    part[threadIdx.x] += v;
-    __syncthreads();
-  }
-  lstart[threadIdx.x] = part[threadIdx.x] - cnt_d;
-  run[threadIdx.x] = part[threadIdx.x] - cnt_d;
+  uint16_t *mine = wcnt + warp * kSortBins;
   uint32_t kr[kSortRounds], vr[kSortRounds];  // all loads of the tile in flight at once
 #pragma unroll
   for (int r = 0; r < kSortRounds; ++r) {
-    const int q = r * kSortThreads + threadIdx.x;
+    const int q = warp * 32 * kSortRounds + r * 32 + lane;
     kr[r] = q < nt ? __ldcs(kin + base + q) : 0u;
-    vr[r] = q < nt ? __ldcs(vin + base + q) : 0u;
+    vr[r] = FIRST ? uint32_t(base + q) : q < nt ? __ldcs(vin + base + q) : 0u;
+  }
+#pragma unroll
+  for (int d = 0; d < kSortBins / 32; ++d) mine[32 * d + lane] = 0;
+  __syncwarp();
+  uint32_t rank[kSortRounds];
+#pragma unroll
+  for (int r = 0; r < kSortRounds; ++r) {
+    const bool valid = warp * 32 * kSortRounds + r * 32 + lane < nt;
+    const unsigned dig = (kr[r] >> shift) & unsigned(ndig - 1);
+    const unsigned peers = digit_peers(dig, nbits, valid);
+    const unsigned before = mine[dig];
+    rank[r] = before + __popc(peers & ((1u << lane) - 1u));
+    __syncwarp();
+    if (valid && (peers >> lane) == 1u) mine[dig] = uint16_t(before + __popc(peers));  // the last of the peers
+    __syncwarp();
+  }
+  __syncthreads();
+  // per digit: the warps' exclusive offsets and the tile's count; then the
+  // counts' exclusive scan over the digits (one digit per thread)
+  uint32_t cnt = 0;
+  if (threadIdx.x < kSortBins) {
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) {
+      const uint32_t c = wcnt[w * kSortBins + threadIdx.x];
+      wcnt[w * kSortBins + threadIdx.x] = uint16_t(cnt);
+      cnt += c;
+    }
+  }
+  uint32_t incl = cnt;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+    if (lane >= off) incl += v;
+  }
+  if (threadIdx.x < kSortBins && lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  if (threadIdx.x < kSortBins) {
+    uint32_t start = incl - cnt;
+    for (int w = 0; w < warp; ++w) start += wsum[w];
+    lstart[threadIdx.x] = start;
+    if (int(threadIdx.x) < ndig)
+      goff[threadIdx.x] = pref[int64_t(blockIdx.x) * ndig + threadIdx.x] +
+                          cbase[int64_t(blockIdx.x / kScanChunk) * ndig + threadIdx.x] + dbase[threadIdx.x] - start;
   }
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < kSortRounds; ++r) {
-    const int q = r * kSortThreads + threadIdx.x;
-    const bool valid = q < nt;
-    const uint32_t k = kr[r];
-    const uint32_t v = vr[r];
-    const unsigned dig = valid ? (k >> shift) & unsigned(ndig - 1) : 0xFFFFFFFFu;
-    const unsigned peers = digit_peers(dig, nbits, valid);
-    const unsigned rank = __popc(peers & ((1u << lane) - 1u));
-    if (valid && rank == 0) wcnt[warp][dig] = __popc(peers);
-    __syncthreads();
-    if (threadIdx.x < ndig) {
-      uint32_t acc = run[threadIdx.x];
-      for (int w = 0; w < kSortThreads / 32; ++w) {
-        const uint32_t c = wcnt[w][threadIdx.x];
-        if (c) {
-          wpre[w][threadIdx.x] = acc;
-          acc += c;
-          wcnt[w][threadIdx.x] = 0;
-        }
-      }
-      run[threadIdx.x] = acc;
-    }
-    __syncthreads();
-    if (valid) {
-      const uint32_t lp = wpre[warp][dig] + rank;
-      skey[lp] = k;
-      sval[lp] = v;
+    if (warp * 32 * kSortRounds + r * 32 + lane < nt) {
+      const unsigned dig = (kr[r] >> shift) & unsigned(ndig - 1);
+      const uint32_t lp = lstart[dig] + mine[dig] + rank[r];
+      skey[lp] = kr[r];
+      sval[lp] = vr[r];
     }
   }
   __syncthreads();
   for (int q = threadIdx.x; q < nt; q += kSortThreads) {
     const uint32_t k = skey[q];
-    const unsigned dig = (k >> shift) & unsigned(ndig - 1);
-    const int64_t dst = int64_t(goff[dig]) + (q - int64_t(lstart[dig]));
+    const uint32_t dst = goff[(k >> shift) & unsigned(ndig - 1)] + uint32_t(q);  // modulo 2^32: np < 2^32
     kout[dst] = k;
     vout[dst] = sval[q];
   }
 }
-
 // particle arrays into the sorted order
 template <class T>
 __global__ void k_part_gather(int64_t np, const uint32_t *__restrict__ perm, const T *__restrict__ x,
@@ -419,6 +460,12 @@ __global__ void k_part_gather(int64_t np, const uint32_t *__restrict__ perm, con
 // ---------------------------------------------------------------------------
 // atomic deposit (warp combining of equal source cells)
 // ---------------------------------------------------------------------------
+// the 8 contributions of source cell (i, j, k) added to the grid
+template <class T>
+__device__ __forceinline__ void add_stencil(const CicGrid<T> &g, int i, int j, int k, const T w[8], T *rho) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) atomicAdd(&rho[grid_at(g.n, i + (c & 1), j + ((c >> 1) & 1), k + (c >> 2))], w[c]);
+}
 template <class T>
 __global__ void __launch_bounds__(256) k_cic_atomic(int64_t np, CicGrid<T> g, const T *__restrict__ x,
                                                     const T *__restrict__ y, const T *__restrict__ z,
@@ -455,10 +502,7 @@ __global__ void __launch_bounds__(256) k_cic_atomic(int64_t np, CicGrid<T> g, co
   // contributions (L2 absorbs the extra atomics).
   const bool combine = sizeof(T) == 4;
   if (combine && runs != 0xFFFFFFFFu) warp_run_sums(w, runs, lane);
-  if (valid && (!combine || ((runs >> lane) & 1u))) {
-#pragma unroll
-    for (int c = 0; c < 8; ++c) atomicAdd(&rho[grid_at(g.n, i + (c & 1), j + ((c >> 1) & 1), k + (c >> 2))], w[c]);
-  }
+  if (valid && (!combine || ((runs >> lane) & 1u))) add_stencil(g, i, j, k, w, rho);
 }
 
 // ---------------------------------------------------------------------------
@@ -470,25 +514,10 @@ __global__ void k_seg_heads(int64_t np, const uint32_t *__restrict__ key, uint32
   flag[q] = (q == 0 || key[q] != key[q - 1]) ? 1u : 0u;
 }
 
-// start[s] of every segment s (scan = exclusive scan of the head flags);
-// start[S] = np and *nseg = S, written by the last particle's thread
-__global__ void k_seg_starts(int64_t np, const uint32_t *__restrict__ key, const uint32_t *__restrict__ scan,
-                             uint32_t *__restrict__ start, uint32_t *__restrict__ nseg) {
-  const int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (q >= np) return;
-  const bool head = q == 0 || key[q] != key[q - 1];
-  if (head) start[scan[q]] = uint32_t(q);
-  if (q == np - 1) {
-    const uint32_t S = scan[q] + (head ? 1u : 0u);
-    start[S] = uint32_t(np);
-    *nseg = S;
-  }
-}
-
 // Per particle, in aligned groups of 32 (one warp each): the contributions
 // summed over each run of equal source cells inside the group (fixed shuffle
-// tree).  A run that starts segment s writes its sums to sums[c * cap + s]
-// and maps its source cell to s; the run at the start of group G that
+// tree).  A run that starts segment s writes its sums to sums[c * cap + s],
+// its first particle to start[s], and maps its source cell to s; the run at the start of group G that
 // continues a segment from earlier groups writes them to carry[c * ngroups + G].
 template <class T>
 __global__ void __launch_bounds__(256) k_seg_partial(int64_t np, CicGrid<T> g, const uint32_t *__restrict__ key,
@@ -496,7 +525,8 @@ __global__ void __launch_bounds__(256) k_seg_partial(int64_t np, CicGrid<T> g, c
                                                      const T *__restrict__ y, const T *__restrict__ z,
                                                      const T *__restrict__ m, int64_t cap, int64_t ngroups,
                                                      T *__restrict__ sums, T *__restrict__ carry,
-                                                     int32_t *__restrict__ cellmap) {
+                                                     int32_t *__restrict__ cellmap, uint32_t *__restrict__ start,
+                                                     uint32_t *__restrict__ nseg) {
   const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   const unsigned lane = threadIdx.x & 31;
   const bool valid = t < np;
@@ -508,6 +538,12 @@ __global__ void __launch_bounds__(256) k_seg_partial(int64_t np, CicGrid<T> g, c
     cic_weights(x[t], y[t], z[t], m[t], g, i, j, k, w);
     kk = key[t];
     head = t == 0 || key[t - 1] != kk;
+    if (head) start[scan[t]] = uint32_t(t);
+    if (t == np - 1) {  // the number of segments; start[S] = np ends the last one
+      const uint32_t S = scan[t] + (head ? 1u : 0u);
+      start[S] = uint32_t(np);
+      *nseg = S;
+    }
   } else {
 #pragma unroll
     for (int c = 0; c < 8; ++c) w[c] = T(0);
