@@ -137,7 +137,7 @@ struct HostPin {
 // level-step launch domains of a segment
 enum Dom {
   DOM_CELLS = 0, DOM_REAL = 1, DOM_GHOST5 = 2, DOM_UPDATE = 3, DOM_BLOCKS = 4, DOM_COMMIT = 5, DOM_RESTRICT = 6,
-  DOM_REFLUX = 7, DOM_COUNT = 8
+  DOM_REFLUX = 7, DOM_UPDATE1 = 8, DOM_COUNT = 9
 };
 
 // a list of segments and, per domain, its tiles: the offset of its tile
@@ -647,6 +647,7 @@ static int dom_size(const Seg &s, int dom) {
     case DOM_BLOCKS: return s.nblk;
     case DOM_COMMIT: return ((s.flags & kSegReflux) ? 5 * s.ncl : 0) + 5 * s.nl;
     case DOM_UPDATE: return 8 * s.nl + ((s.flags & kSegReflux) ? 5 * s.ncl : 0);
+    case DOM_UPDATE1: return 8 * s.nl + ((s.flags & kSegReflux) ? s.ncl : 0);
     case DOM_REFLUX: return (s.flags & kSegReflux) ? 5 * s.ncl : 0;
     default: return (s.flags & kSegRestrict) ? 5 * s.nl : 0;
   }
@@ -804,7 +805,7 @@ static StepArgs<T> step_args(amr_mesh *h, bool device_dt, double dt) {
 
 // persistent grid: enough blocks to fill the GPU once, never more than tiles.
 // smem: bytes of dynamic shared memory per thread; per_tile: blocks that share a
-// tile (3: one per axis)
+// tile (3: one per axis, 5: one per variable)
 template <class T>
 static void run_list(amr_mesh *h, int kid, void (*kern)(StepArgs<T>), StepArgs<T> a,
                      const SegList &L, int dom, size_t smem = 0, int per_tile = 1) {
@@ -887,6 +888,20 @@ static void run_prolong(amr_mesh *h, StepArgs<T> a, const SegList &L, const SegL
   launch(h, K_PROLONG, k_prolong<T>, dim3(unsigned(grid)), dim3(unsigned(h->tile_size)), a, p);
 }
 
+// Up to this many local cells a list does not fill the GPU, and a level step lasts
+// as long as its kernels' chains of loads and arithmetic: it takes the kernels with
+// more threads and less per thread, k_update_small and, in FP32, a solve per face
+// (k_flux).  Times of a step, these kernels against the others:
+//   FP64  levels of 2-15 thousand cells (random mesh 3-6) 0.308 against 0.333 ms,
+//         a level of 33 thousand 41.1 us both, levels of 25-72 thousand 118 against
+//         111 us (Sod 5-6), one of 262 thousand 162 against 146 us
+//   FP32  random mesh 3-6 0.202 against 0.280 ms, Sod 5-6 53 against 66 us, levels
+//         of 15-100 thousand (Sedov 6-9) 0.234 against 0.310 ms, one of 262
+//         thousand 48.6 against 42.7 us: every face is solved twice there, but
+//         nothing is stored in between
+template <class T>
+constexpr int kSmallList = sizeof(T) == 8 ? 16384 : 131072;
+
 template <class T>
 static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double dt, const SegList **pend) {
   if (L.nseg == 0) return;
@@ -915,19 +930,30 @@ static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double d
     // new leaf states from the scratch into U, with reflux sums and restriction
     run_list(h, K_COMMIT, k_commit_post<T>, a, L, DOM_COMMIT);
     return;
-  } else if constexpr (sizeof(T) == 4) {
-    // FP32: primitives recomputed inside the predictor; each leaf cell solves
-    // its six faces and updates itself
+  }
+  const bool small = L.ls <= kSmallList<T>;
+  if constexpr (sizeof(T) == 4) {
     run_list(h, K_PREDICT, k_predict_u, a, L, DOM_CELLS);
-    run_list(h, K_FLUX, k_flux_update, a, L, DOM_REAL, 20);
-    if (L.ntile[DOM_REFLUX]) *pend = &L;
+    if (!small) {
+      // primitives recomputed inside the predictor; each leaf cell solves its six
+      // faces and updates itself
+      run_list(h, K_FLUX, k_flux_update, a, L, DOM_REAL, 20);
+      if (L.ntile[DOM_REFLUX]) *pend = &L;
+      return;
+    }
   } else {
     // FP64: every predictor and every face solve exactly once
     run_list(h, K_PRIM, k_ghost_prim, a, L, DOM_CELLS, 16);
     run_list(h, K_PREDICT, k_predict, a, L, DOM_CELLS);
-    run_list(h, K_FLUX, k_flux, a, L, DOM_CELLS, 0, 3);
-    run_list(h, K_UPDATE, k_update, a, L, DOM_UPDATE, 40);
   }
+  run_list(h, K_FLUX, k_flux<T>, a, L, DOM_CELLS, 0, 3);
+  if constexpr (sizeof(T) == 8) {
+    if (!small) {
+      run_list(h, K_UPDATE, k_update, a, L, DOM_UPDATE, 40);
+      return;
+    }
+  }
+  run_list(h, K_UPDATE, k_update_small<T>, a, L, DOM_UPDATE1, sizeof(T), 5);
 }
 
 // One level step of a list.  *pend: a list whose reflux sums are still to be

@@ -58,6 +58,47 @@ __host__ __device__ __forceinline__ uint64_t mul_bits(uint64_t x, uint64_t y) {
   return (uint64_t(hi) << 32) | m;
 }
 
+// Sum of six doubles (bit k of NEG: the k-th is subtracted), rounded once, on the
+// integer pipes: the mantissas, shifted to the largest exponent with 7 bits below
+// its last place, add up in 64 bits (some 120 instructions; 5 additions hold the
+// FP64 pipe for 80 cycles of an SM).  Each term loses less than 2^-7 units in the
+// last place of the largest, the sum is then rounded to the nearest double:
+// against the exact sum at most 0.05 of those units more than one rounding, where
+// a chain of five additions rounds five times.  As in the products, what lies below
+// the normal range is zero.  `ok`: false where an operand is infinite, NaN or too
+// large for the sum; the caller then adds them on the FP64 pipe.
+template <unsigned NEG>
+__host__ __device__ __forceinline__ uint64_t sum6_bits(const uint64_t (&x)[6], bool &ok) {
+  uint32_t top = 0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const uint32_t e = uint32_t(x[k] >> 32) & 0x7FF00000u;
+    top = e > top ? e : top;
+  }
+  ok = top < (2042u << 20);
+  uint64_t sum = 0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const uint32_t h = uint32_t(x[k] >> 32), e = h & 0x7FF00000u;
+    const uint64_t m = e ? ((x[k] & 0xFFFFFFFFFFFFFull) | (uint64_t(1) << 52)) << 7 : 0;
+    const uint32_t d = (top - e) >> 20;
+    const uint64_t t = m >> (d < 63 ? d : 63);
+    const bool minus = (h >> 31) != ((NEG >> k) & 1u);
+    sum = minus ? sum - t : sum + t;
+  }
+  const uint64_t neg = sum >> 63, a = neg ? 0 - sum : sum;
+  if (a == 0) return 0;
+#ifdef __CUDA_ARCH__
+  const int z = __clzll((long long)a);
+#else
+  const int z = __builtin_clzll(a);
+#endif
+  const uint64_t n = a << z;
+  const uint64_t r = (n >> 11) + ((n >> 10) & 1);
+  const int e = int(top >> 20) + 3 - z;  // of the sum, less one (the mantissa's leading bit adds it)
+  return e < 0 ? 0 : (neg << 63) | ((uint64_t(e) << 52) + r);
+}
+
 #ifndef FP64_INT_HOST
 __device__ __forceinline__ double mul_int(double x, double y) {
   return __longlong_as_double(
@@ -74,6 +115,19 @@ __device__ __forceinline__ double normal_or_zero(double x) {
 }
 __device__ __forceinline__ double mul_fp64_0(double x, double y) {
   return normal_or_zero(__dmul_rn(normal_or_zero(x), normal_or_zero(y)));
+}
+
+template <unsigned NEG>
+__device__ __forceinline__ double sum6_int(double a, double b, double c, double d, double e, double f) {
+  const uint64_t x[6] = {uint64_t(__double_as_longlong(a)), uint64_t(__double_as_longlong(b)),
+                         uint64_t(__double_as_longlong(c)), uint64_t(__double_as_longlong(d)),
+                         uint64_t(__double_as_longlong(e)), uint64_t(__double_as_longlong(f))};
+  bool ok;
+  const uint64_t s = sum6_bits<NEG>(x, ok);
+  if (ok) return __longlong_as_double((long long)s);
+  const double ab = __dadd_rn(NEG & 1 ? -a : a, NEG & 2 ? -b : b), cd = __dadd_rn(NEG & 4 ? -c : c, NEG & 8 ? -d : d),
+               ef = __dadd_rn(NEG & 16 ? -e : e, NEG & 32 ? -f : f);
+  return __dadd_rn(__dadd_rn(ab, cd), ef);
 }
 
 // x in [2^-E, 2^E)

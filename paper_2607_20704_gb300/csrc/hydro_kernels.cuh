@@ -168,25 +168,40 @@ __device__ __forceinline__ SegCtx<T> seg_ctx(const StepArgs<T> &a, const Seg &s)
   return c;
 }
 
-// persistent loop over the launch's tiles: body(ctx, item) for every item of
-// the tile that lies inside the segment's domain of `size(ctx)` items
-template <class T, class Size, class Body>
-__device__ __forceinline__ void tile_loop(const StepArgs<T> &a, Size size, Body body) {
+// the segment's context; false: nothing to do (a finished member)
+template <class T>
+__device__ __forceinline__ bool open_segment(const StepArgs<T> &a, int seg, SegCtx<T> &s) {
+  const Seg sg = seg_at(a.tiles, seg);
+  if (a.mact && !__ldg(a.mact + sg.member)) return false;
+  s = seg_ctx(a, sg);
+#ifdef AMR_CHECKED
+  // the segment's local cells must fit the scratch arrays
+  if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
+    atomicOr(a.err, kErrIndex);
+    return false;
+  }
+#endif
+  return true;
+}
+
+// persistent loop over the launch's tiles: body(ctx, item) for every thread of a
+// tile's block, also beyond the segment's items (bodies work by whole warps)
+template <class T, class Body>
+__device__ __forceinline__ void warp_tile_loop(const StepArgs<T> &a, Body body) {
   for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
     const Tile td = tile_at(a.tiles, ti);
-    const Seg sg = seg_at(a.tiles, td.seg);
-    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
-    const SegCtx<T> sc = seg_ctx(a, sg);
-#ifdef AMR_CHECKED
-    // the segment's local cells must fit the scratch arrays
-    if (sc.base < 0 || sc.base + 8 * (sc.nl + sc.ncl) > a.LS) {
-      atomicOr(a.err, kErrIndex);
-      continue;
-    }
-#endif
-    const int item = td.start + threadIdx.x;
-    if (item < size(sc)) body(sc, item);
+    SegCtx<T> s;
+    if (open_segment(a, td.seg, s)) body(s, td.start + int(threadIdx.x));
   }
+}
+
+// the same for every item of the tile that lies inside the segment's domain of
+// `size(ctx)` items
+template <class T, class Size, class Body>
+__device__ __forceinline__ void tile_loop(const StepArgs<T> &a, Size size, Body body) {
+  warp_tile_loop(a, [&](const SegCtx<T> &s, int item) {
+    if (item < size(s)) body(s, item);
+  });
 }
 
 // extended oct index of local oct index q, and back
@@ -226,9 +241,15 @@ template <class T>
 __device__ __forceinline__ void reflux_sum(const StepArgs<T> &a, int v, int g) {
   const T *cv = a.C + v * a.CS + 24 * int64_t(g);
   T *Rv = a.Rc + v * int64_t(a.NC) + g;
+  constexpr int W = 16 / sizeof(T);  // 16 bytes per load: a ghost oct's slots are 192 (96) bytes in a row
+  struct alignas(16) Slots {
+    T x[W];
+  } sl[24 / W];
+#pragma unroll
+  for (int k = 0; k < 24 / W; ++k) sl[k] = reinterpret_cast<const Slots *>(cv)[k];
   T acc = *Rv;
 #pragma unroll
-  for (int k = 0; k < 24; ++k) acc += cv[k];
+  for (int k = 0; k < 24; ++k) acc += sl[k / W].x[k % W];
   *Rv = acc;
 }
 
@@ -361,20 +382,9 @@ __device__ __forceinline__ void prim_at(const StepArgs<T> &a, const SegCtx<T> &s
 // its cells.
 __global__ void __launch_bounds__(512, 3) k_ghost_prim(StepArgs<double> a) {
   extern __shared__ double slopes[];  // [5 d + v][oct of the block], 16 bytes per thread
-  const int nq = blockDim.x >> 3;
-  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tiles, ti);
-    const Seg sg = seg_at(a.tiles, td.seg);
-    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
-    const SegCtx<double> s = seg_ctx(a, sg);
-#ifdef AMR_CHECKED
-    if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
-      atomicOr(a.err, kErrIndex);
-      continue;
-    }
-#endif
-    const int t = td.start + threadIdx.x;
-    const int q = t >> 3, c = t & 7, qb = threadIdx.x >> 3;
+  const int qb = threadIdx.x >> 3, nq = blockDim.x >> 3;
+  warp_tile_loop(a, [&](const SegCtx<double> &s, int t) {
+    const int q = t >> 3, c = t & 7;
     const bool on = t < 8 * (s.nl + s.ncl), ghost = on && q >= s.nl;
     const int cs = s.clo + (q - s.nl);
     const int64_t g = 8 * int64_t(ext_of_local(a, s, q)) + c;
@@ -419,7 +429,7 @@ __global__ void __launch_bounds__(512, 3) k_ghost_prim(StepArgs<double> a) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) a.W[v * a.LS + o] = w[v];
     }
-  }
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -498,27 +508,28 @@ __device__ __forceinline__ double shfl_xor_f64(unsigned mask, double x, int lane
   return __hiloint2double(hi, lo);
 }
 __global__ void k_predict(StepArgs<double> a) {
-  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tiles, ti);
-    const Seg sg = seg_at(a.tiles, td.seg);
-    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
-    const SegCtx<double> s = seg_ctx(a, sg);
-#ifdef AMR_CHECKED
-    if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
-      atomicOr(a.err, kErrIndex);
-      continue;
-    }
-#endif
-    const int t = td.start + threadIdx.x;  // tiles start at multiples of 8: octs are whole
+  warp_tile_loop(a, [&](const SegCtx<double> &s, int t) {  // tiles start at multiples of 8: octs are whole
     const bool on = t < 8 * (s.nl + s.ncl);
     const unsigned lanes = __ballot_sync(0xFFFFFFFFu, on);
-    if (!on) continue;
+    if (!on) return;
     const int e = ext_of_local(a, s, t >> 3);
     const int c = t & 7;
     const int o = s.base + t;
+    // the three outer neighbours, or the cell itself (outer ring of a ghost oct,
+    // slopes never used): all addresses before the first wait
+    int out[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int to = nbr_local(a, s, t, e, c, d, (c >> d) & 1);
+      out[d] = to >= 0 ? s.base + to : o;
+    }
     double w[5], dw[3][5], ws[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) w[v] = a.W[v * a.LS + o];
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int v = 0; v < 5; ++v) dw[d][v] = a.W[v * a.LS + out[d]];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const int bit = 1 << d;
@@ -534,19 +545,12 @@ __global__ void k_predict(StepArgs<double> a) {
       }
       const double got = shfl_xor_f64(lanes, w[4], bit);
       in[4] = (up ? w[4] : got) - (up ? got : w[4]);
-      const int to = nbr_local(a, s, t, e, c, d, up ? 1 : 0);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        dw[d][v] = 0.0;  // outer ring of a ghost oct: never used
-        if (to >= 0) {
-          const double wo = a.W[v * a.LS + s.base + to];
-          dw[d][v] = minmod((up ? wo : w[v]) - (up ? w[v] : wo), in[v]);
-        }
-      }
+      for (int v = 0; v < 5; ++v) dw[d][v] = minmod((up ? dw[d][v] : w[v]) - (up ? w[v] : dw[d][v]), in[v]);
     }
     predictor(s, w, dw, ws);
     store_q(a, o, ws, dw);
-  }
+  });
 }
 
 // FP32: primitives derived from U directly (no W array): the cell's own and its
@@ -554,21 +558,10 @@ __global__ void k_predict(StepArgs<double> a) {
 // its oct (four conversions and 20 gathered loads per cell instead of seven
 // and 35)
 __global__ void __launch_bounds__(512, 3) k_predict_u(StepArgs<float> a) {
-  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tiles, ti);
-    const Seg sg = seg_at(a.tiles, td.seg);
-    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
-    const SegCtx<float> s = seg_ctx(a, sg);
-#ifdef AMR_CHECKED
-    if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
-      atomicOr(a.err, kErrIndex);
-      continue;
-    }
-#endif
-    const int t = td.start + threadIdx.x;  // tiles start at multiples of 8: octs are whole
+  warp_tile_loop(a, [&](const SegCtx<float> &s, int t) {  // tiles start at multiples of 8: octs are whole
     const bool on = t < 8 * (s.nl + s.ncl);
     const unsigned lanes = __ballot_sync(0xFFFFFFFFu, on);
-    if (!on) continue;
+    if (!on) return;
     const int e = ext_of_local(a, s, t >> 3);
     const int c = t & 7;
     float w[5], dw[3][5], ws[5];
@@ -589,7 +582,7 @@ __global__ void __launch_bounds__(512, 3) k_predict_u(StepArgs<float> a) {
     }
     predictor(s, w, dw, ws);
     store_q(a, s.base + t, ws, dw);
-  }
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -761,24 +754,18 @@ __device__ __forceinline__ int64_t reflux_slot(int D, int clo, int nl, int gq, i
 // axes are consecutive blocks: the faces of a small level are solved at once
 // (one after the other they are a chain of three solves, which bounds a level
 // that does not fill the GPU), and a large level finds the cells' states in L2.
-__global__ void k_flux(StepArgs<double> a) {
+template <class T>
+__global__ void k_flux(StepArgs<T> a) {
   for (int tb = blockIdx.x; tb < 3 * a.tiles.ntiles; tb += gridDim.x) {
     const int ti = tb / 3, D = tb - 3 * ti;
     const Tile td = tile_at(a.tiles, ti);
-    const Seg sg = seg_at(a.tiles, td.seg);
-    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
-    const SegCtx<double> s = seg_ctx(a, sg);
-#ifdef AMR_CHECKED
-    if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
-      atomicOr(a.err, kErrIndex);
-      continue;
-    }
-#endif
+    SegCtx<T> s;
+    if (!open_segment(a, td.seg, s)) continue;
     const int t = td.start + threadIdx.x;
     if (t >= 8 * (s.nl + s.ncl)) continue;
     const int q = t >> 3, c = t & 7;
     const bool real = q < s.nl;
-    double F[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    T F[5] = {T(0), T(0), T(0), T(0), T(0)};
     const int tn = nbr_local(a, s, t, ext_of_local(a, s, q), c, D, 1);
     if (tn >= 0) {
       const bool nreal = (tn >> 3) < s.nl;
@@ -789,10 +776,10 @@ __global__ void k_flux(StepArgs<double> a) {
           // ghost on the minus side: its plus face (sigma -1)
           const int64_t gslot = real ? reflux_slot(D, s.clo, s.nl, tn >> 3, 2 * D, c)
                                      : reflux_slot(D, s.clo, s.nl, t >> 3, 2 * D + 1, c);
-          const double sg8 = real ? 1.0 : -1.0;
+          const T sg8 = real ? T(1) : T(-1);
 #pragma unroll
           for (int v = 0; v < 5; ++v)
-            a.C[v * a.CS + checked(gslot, 0, a.CS, a.err)] = (sg8 * s.dtdx) * F[v] / 8.0;
+            a.C[v * a.CS + checked(gslot, 0, a.CS, a.err)] = (sg8 * s.dtdx) * F[v] / T(8);
         }
       }
     }
@@ -801,28 +788,31 @@ __global__ void k_flux(StepArgs<double> a) {
   }
 }
 
-// U <- (U + dt/dx sum_d (F_d- - F_d+)) + R on leaf cells; R <- 0
+// sum over the axes of F(minus face) - F(plus face) of one variable; FP64 on the
+// integer pipes (five additions hold the FP64 pipe for 80 cycles of an SM), rounded
+// once
+__device__ __forceinline__ double flux_sum(double xm, double xp, double ym, double yp, double zm, double zp) {
+  return sum6_int<0x2A>(xm, xp, ym, yp, zm, zp);
+}
+__device__ __forceinline__ float flux_sum(float xm, float xp, float ym, float yp, float zm, float zp) {
+  return ((xm - xp) + (ym - yp)) + (zm - zp);
+}
+
+// new state (u + dt/dx dF) + R of variable v of leaf cell g, dF its flux sum, rs
+// the slot of its pending reflux R (or -1); R <- 0
 template <class T>
-__device__ __forceinline__ void new_state(const StepArgs<T> &a, const SegCtx<T> &s, int g, const T (&dx)[5],
-                                          const T (&dy)[5], const T (&dz)[5], T (&un)[5]) {
-  const int rs = int(checked(__ldg(a.rslot + g), -1, a.NC, a.err, -1));
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    T u = a.U[v * a.S + g] + s.dtdx * ((dx[v] + dy[v]) + dz[v]);
-    if (rs >= 0) {
-      T *Rv = a.Rc + v * int64_t(a.NC) + rs;
-      u = u + *Rv;
-      *Rv = T(0);
-    }
-    un[v] = u;
+__device__ __forceinline__ T new_state(const StepArgs<T> &a, const SegCtx<T> &s, int v, int g, T u, int rs, T dF) {
+  u = u + s.dtdx * dF;
+  if (rs >= 0) {
+    T *Rv = a.Rc + v * int64_t(a.NC) + rs;
+    u = u + *Rv;
+    *Rv = T(0);
   }
+  return u;
 }
 template <class T>
-__device__ __forceinline__ void update_cell(const StepArgs<T> &a, const SegCtx<T> &s, int g, const T (&dx)[5],
-                                            const T (&dy)[5], const T (&dz)[5], T (&un)[5]) {
-  new_state(a, s, g, dx, dy, dz, un);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) a.U[v * a.S + g] = un[v];
+__device__ __forceinline__ int reflux_of(const StepArgs<T> &a, int g) {
+  return int(checked(__ldg(a.rslot + g), -1, a.NC, a.err, -1));
 }
 
 // father cell (index in its oct) of the oct with internal key k
@@ -830,78 +820,102 @@ __device__ __forceinline__ int father_cell(uint64_t k) {
   return int((ikey_x(k) & 1) | ((ikey_y(k) & 1) << 1) | ((ikey_z(k) & 1) << 2));
 }
 
-// Restriction by a warp of the octs of its 32 cells onto their father cells,
-// (sum of the 8 children in child order) / 8: the lanes' new states u (where on)
-// go through the warp's rows sm[v stride + lane], one lane per (oct, variable)
+// restriction of local oct q, variable v: father cell = (sum of the 8 children's
+// new states u[0..8) in child order) / 8
 template <class T>
-__device__ __forceinline__ void restrict_octs(const StepArgs<T> &a, const SegCtx<T> &s, int t, int lane, bool on,
-                                              const T (&u)[5], T *sm, int stride) {
-  __syncwarp();
-  if (on) {
+__device__ __forceinline__ void restrict_oct(const StepArgs<T> &a, const SegCtx<T> &s, int q, int v, const T *u) {
+  const int o = s.lo + q;
+  const int fc = father_cell(__ldg(a.key + o));
+  const int f = int(checked(__ldg(a.father + o), 0, a.N, a.err));
+  T sum = T(0);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) sm[v * stride + lane] = u[v];
-  }
-  __syncwarp();
-  const int q = ((t - lane) >> 3) + (lane & 3), v = lane >> 2;  // local oct, variable
-  if (v < 5 && q < s.nl) {
-    const int o = s.lo + q;
-    const int fc = father_cell(__ldg(a.key + o));
-    const int f = int(checked(__ldg(a.father + o), 0, a.N, a.err));
-    const T *src = sm + v * stride + 8 * (lane & 3);
-    T sum = T(0);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) sum += src[c];
-    a.U[v * a.S + 8 * int64_t(f) + fc] = sum * T(0.125);
-  }
-  __syncwarp();
+  for (int c = 0; c < 8; ++c) sum += u[c];
+  a.U[v * a.S + 8 * int64_t(f) + fc] = sum * T(0.125);
 }
 
-// FP64: the last pass of a level step: new states of the leaf cells, the
-// restriction of the same warp's octs and, beyond the cells, the reflux sums of
-// the level's ghost octs.  They touch disjoint data: the level's cells, the
-// coarser level's split cells, the pending reflux of its leaf cells.
+// The last pass of a level step: new states of the leaf cells, the restriction of
+// their octs and, beyond the cells, the reflux sums of the level's ghost octs.
+// They touch disjoint data: the level's cells, the coarser level's split cells,
+// the pending reflux of its leaf cells.
+
+// FP64, a list that fills the GPU: a thread per cell, one variable after the other.
+// Sedov 7-10 / clustered 6-9, us per coarse step: 458 / 275; the sums on the FP64
+// pipe 481 / 385; all five variables unrolled 455 / 367; a thread per (cell,
+// variable) 672 / 463 (the cell's five index loads are repeated).  A branch around
+// the sum for warps of gas at rest: 441 / 441.
 // domain: 8 nl, + 5 ncl (if kSegReflux)
-__global__ void __launch_bounds__(512, 3) k_update(StepArgs<double> a) {
+__global__ void __launch_bounds__(512, 2) k_update(StepArgs<double> a) {
   extern __shared__ double update_smem[];  // the block's new states [5][threads]
   const int lane = threadIdx.x & 31;
-  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tiles, ti);
-    const Seg sg = seg_at(a.tiles, td.seg);
-    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
-    const SegCtx<double> s = seg_ctx(a, sg);
-#ifdef AMR_CHECKED
-    if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
-      atomicOr(a.err, kErrIndex);
-      continue;
-    }
-#endif
-    const int t = td.start + threadIdx.x;
-    const bool on = t < 8 * s.nl;
-    double u[5];
-    if (on) {
-      const int e = s.lo + (t >> 3), c = t & 7;
-      if (cell_is_split(a, s, t)) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + 8 * e + c];
-      } else {
-        const int o = s.base + t;
-        const int om[3] = {s.base + nbr_local(a, s, t, e, c, 0, 0), s.base + nbr_local(a, s, t, e, c, 1, 0),
-                           s.base + nbr_local(a, s, t, e, c, 2, 0)};
-        double dx[5], dy[5], dz[5];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          dx[v] = a.F[(0 + v) * a.LS + om[0]] - a.F[(0 + v) * a.LS + o];
-          dy[v] = a.F[(5 + v) * a.LS + om[1]] - a.F[(5 + v) * a.LS + o];
-          dz[v] = a.F[(10 + v) * a.LS + om[2]] - a.F[(10 + v) * a.LS + o];
+  warp_tile_loop(a, [&](const SegCtx<double> &s, int t) {
+    if (t < 8 * s.nl) {
+      const int e = s.lo + (t >> 3), c = t & 7, g = 8 * e + c;
+      const bool leaf = !cell_is_split(a, s, t);
+      int mx = 0, my = 0, mz = 0, rs = -1;
+      if (leaf) {
+        mx = nbr_local(a, s, t, e, c, 0, 0);
+        my = nbr_local(a, s, t, e, c, 1, 0);
+        mz = nbr_local(a, s, t, e, c, 2, 0);
+        rs = reflux_of(a, g);
+      }
+#pragma unroll 1
+      for (int v = 0; v < 5; ++v) {
+        double u = a.U[v * a.S + g];
+        if (leaf) {
+          const double *Fx = a.F + v * a.LS + s.base, *Fy = Fx + 5 * a.LS, *Fz = Fy + 5 * a.LS;
+          u = new_state(a, s, v, g, u, rs, flux_sum(Fx[mx], Fx[t], Fy[my], Fy[t], Fz[mz], Fz[t]));
+          a.U[v * a.S + g] = u;
         }
-        update_cell(a, s, 8 * e + c, dx, dy, dz, u);
+        if (s.flags & kSegRestrict) update_smem[v * blockDim.x + threadIdx.x] = u;
       }
     } else if ((s.flags & kSegReflux) && t - 8 * s.nl < 5 * s.ncl) {
       const int q = t - 8 * s.nl, v = q / s.ncl;
       reflux_sum(a, v, s.clo + (q - v * s.ncl));
     }
-    if (s.flags & kSegRestrict)
-      restrict_octs(a, s, t, lane, on, u, update_smem + threadIdx.x - lane, int(blockDim.x));
+    if (s.flags & kSegRestrict) {  // a lane per (oct, variable)
+      __syncwarp();
+      const int q = ((t - lane) >> 3) + (lane & 3), v = lane >> 2;
+      if (v < 5 && q < s.nl)
+        restrict_oct(a, s, q, v, update_smem + v * blockDim.x + (threadIdx.x - lane) + 8 * (lane & 3));
+      __syncwarp();
+    }
+  });
+}
+
+// A small list: a thread per (cell, variable), a tile's five variables in
+// consecutive blocks (five times the threads and a fifth of the chain).
+// domain: 8 nl, + ncl (if kSegReflux)
+template <class T>
+__global__ void k_update_small(StepArgs<T> a) {
+  extern __shared__ __align__(8) unsigned char update_bytes[];
+  T *sm = reinterpret_cast<T *>(update_bytes);  // the block's new states
+  const int lane = threadIdx.x & 31;
+  for (int tb = blockIdx.x; tb < 5 * a.tiles.ntiles; tb += gridDim.x) {
+    const int ti = tb / 5, v = tb - 5 * ti;
+    const Tile td = tile_at(a.tiles, ti);
+    SegCtx<T> s;
+    if (!open_segment(a, td.seg, s)) continue;
+    const int t = td.start + threadIdx.x;
+    if (t < 8 * s.nl) {
+      const int e = s.lo + (t >> 3), c = t & 7, g = 8 * e + c;
+      T u = a.U[v * a.S + g];
+      if (!cell_is_split(a, s, t)) {
+        const T *Fx = a.F + v * a.LS + s.base, *Fy = Fx + 5 * a.LS, *Fz = Fy + 5 * a.LS;
+        const int mx = nbr_local(a, s, t, e, c, 0, 0), my = nbr_local(a, s, t, e, c, 1, 0),
+                  mz = nbr_local(a, s, t, e, c, 2, 0);
+        u = new_state(a, s, v, g, u, reflux_of(a, g), flux_sum(Fx[mx], Fx[t], Fy[my], Fy[t], Fz[mz], Fz[t]));
+        a.U[v * a.S + g] = u;
+      }
+      sm[threadIdx.x] = u;
+    } else if ((s.flags & kSegReflux) && t - 8 * s.nl < s.ncl) {
+      reflux_sum(a, v, s.clo + (t - 8 * s.nl));
+    }
+    if (s.flags & kSegRestrict) {
+      __syncwarp();
+      const int q = ((t - lane) >> 3) + lane;
+      if (lane < 4 && q < s.nl) restrict_oct(a, s, q, v, sm + (threadIdx.x - lane) + 8 * lane);
+      __syncwarp();
+    }
   }
 }
 
@@ -944,36 +958,38 @@ __device__ __forceinline__ void faces_dir(const StepArgs<float> &a, const SegCtx
 __global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<float> a) {
   extern __shared__ float flux_smem[];  // the block's new states [5][threads]
   const int lane = threadIdx.x & 31;
-  for (int ti = blockIdx.x; ti < a.tiles.ntiles; ti += gridDim.x) {
-    const Tile td = tile_at(a.tiles, ti);
-    const Seg sg = seg_at(a.tiles, td.seg);
-    if (a.mact && !__ldg(a.mact + sg.member)) continue;  // finished member
-    const SegCtx<float> s = seg_ctx(a, sg);
-#ifdef AMR_CHECKED
-    if (s.base < 0 || s.base + 8 * (s.nl + s.ncl) > a.LS) {
-      atomicOr(a.err, kErrIndex);
-      continue;
-    }
-#endif
-    const int t = td.start + threadIdx.x;
-    const bool on = t < 8 * s.nl;
-    float u[5];
-    if (on) {
-      const int e = s.lo + (t >> 3), c = t & 7;
+  warp_tile_loop(a, [&](const SegCtx<float> &s, int t) {
+    if (t < 8 * s.nl) {
+      const int e = s.lo + (t >> 3), c = t & 7, g = 8 * e + c;
+      float u[5];
       if (cell_is_split(a, s, t)) {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + 8 * e + c];
+        for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + g];
       } else {
         float dx[5], dy[5], dz[5];
         faces_dir<0>(a, s, t, e, c, dx);
         faces_dir<1>(a, s, t, e, c, dy);
         faces_dir<2>(a, s, t, e, c, dz);
-        update_cell(a, s, 8 * e + c, dx, dy, dz, u);
+        const int rs = reflux_of(a, g);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          u[v] = new_state(a, s, v, g, a.U[v * a.S + g], rs, (dx[v] + dy[v]) + dz[v]);
+          a.U[v * a.S + g] = u[v];
+        }
+      }
+      if (s.flags & kSegRestrict) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) flux_smem[v * blockDim.x + threadIdx.x] = u[v];
       }
     }
-    if (s.flags & kSegRestrict)
-      restrict_octs(a, s, t, lane, on, u, flux_smem + threadIdx.x - lane, int(blockDim.x));
-  }
+    if (s.flags & kSegRestrict) {  // the warp's octs, a lane per (oct, variable)
+      __syncwarp();
+      const int q = ((t - lane) >> 3) + (lane & 3), v = lane >> 2;
+      if (v < 5 && q < s.nl)
+        restrict_oct(a, s, q, v, flux_smem + v * blockDim.x + (threadIdx.x - lane) + 8 * (lane & 3));
+      __syncwarp();
+    }
+  });
 }
 
 // Restriction alone (of a state that was written): father cell = (sum of the 8
@@ -982,15 +998,8 @@ template <class T>
 __global__ void k_restrict(StepArgs<T> a) {
   tile_loop(a, [](const SegCtx<T> &s) { return (s.flags & kSegRestrict) ? 5 * s.nl : 0; },
             [&](const SegCtx<T> &s, int r) {
-              const int v = r / s.nl;
-              const int o = s.lo + (r - v * s.nl);
-              const int fc = father_cell(__ldg(a.key + o));
-              const int f = int(checked(__ldg(a.father + o), 0, a.N, a.err));
-              const T *src = a.U + v * a.S + 8 * int64_t(o);
-              T sum = T(0);
-#pragma unroll
-              for (int c = 0; c < 8; ++c) sum += src[c];
-              a.U[v * a.S + 8 * int64_t(f) + fc] = sum * T(0.125);
+              const int v = r / s.nl, q = r - v * s.nl;
+              restrict_oct(a, s, q, v, a.U + v * a.S + 8 * int64_t(s.lo + q));
             });
 }
 

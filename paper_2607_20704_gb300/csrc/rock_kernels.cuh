@@ -430,23 +430,15 @@ __global__ void __launch_bounds__(Rock<NS>::THREADS, Rock<NS>::template min_bloc
       const int pf[3] = {xi < IN - 1 ? gi + 1 : IC + yi + IN * zi,
                          yi < IN - 1 ? gi + IN : IC + xi + IN * zi,
                          zi < IN - 1 ? gi + IN * IN : IC + xi + IN * yi};
-      T du[3][5];
-#pragma unroll
-      for (int D = 0; D < 3; ++D)
-#pragma unroll
-        for (int v = 0; v < 5; ++v) du[D][v] = sF[(5 * D + v) * FS + gi] - sF[(5 * D + v) * FS + pf[D]];
       const int64_t g = 8 * int64_t(e) + c;
-      const int rs = int(checked(__ldg(a.rslot + g), -1, a.NC, a.err, -1));
+      const int rs = reflux_of(a, int(g));
       T *out = a.W + s.base + 8 * (e - s.lo) + c;
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        T u = __ldg(a.U + v * a.S + g) + s.dtdx * ((du[0][v] + du[1][v]) + du[2][v]);
-        if (rs >= 0) {
-          T *Rv = a.Rc + v * int64_t(a.NC) + rs;
-          u = u + *Rv;
-          *Rv = T(0);
-        }
-        out[v * a.LS] = u;
+        const T *Fv = sF + v * FS;
+        const T dF = flux_sum(Fv[gi], Fv[pf[0]], Fv[5 * FS + gi], Fv[5 * FS + pf[1]], Fv[10 * FS + gi],
+                              Fv[10 * FS + pf[2]]);
+        out[v * a.LS] = new_state(a, s, v, g, __ldg(a.U + v * a.S + g), rs, dF);
       }
     }
     __syncthreads();
@@ -665,18 +657,17 @@ __global__ void __launch_bounds__(Sweep<NS>::THREADS) k_sweep(StepArgs<T> a, con
             if (ctype[x + E * (y + E * zu)] != (kCellLeaf | kCellOwn)) continue;
             int e, c;
             cube_cell<T, NS>(a, octs, x, y, zu, o0, o1, e, c);
-            T du[3][5];
+            T dF[5];
 #pragma unroll
-            for (int v = 0; v < 5; ++v) {
-              du[0][v] = sFx[v * FNP + (x - 2) + FP * (y - 2)] - sFx[v * FNP + (x - 1) + FP * (y - 2)];
-              du[1][v] = sFy[v * FNP + (y - 2) + FP * (x - 2)] - sFy[v * FNP + (y - 1) + FP * (x - 2)];
-              du[2][v] = Fzl[v * ZF + (x - 2) + IN * (y - 2)] - Fzc[v * ZF + (x - 2) + IN * (y - 2)];
-            }
+            for (int v = 0; v < 5; ++v)
+              dF[v] = flux_sum(sFx[v * FNP + (x - 2) + FP * (y - 2)], sFx[v * FNP + (x - 1) + FP * (y - 2)],
+                               sFy[v * FNP + (y - 2) + FP * (x - 2)], sFy[v * FNP + (y - 1) + FP * (x - 2)],
+                               Fzl[v * ZF + (x - 2) + IN * (y - 2)], Fzc[v * ZF + (x - 2) + IN * (y - 2)]);
             const int t = 8 * (e - s.lo) + c;
-            T un[5];  // into the scratch: other blocks may still read the old state
-            new_state(a, s, 8 * e + c, du[0], du[1], du[2], un);
+            const int rs = reflux_of(a, 8 * e + c);
 #pragma unroll
-            for (int v = 0; v < 5; ++v) a.W[v * int64_t(a.LS) + s.base + t] = un[v];
+            for (int v = 0; v < 5; ++v)  // into the scratch: other blocks may still read the old state
+              a.W[v * int64_t(a.LS) + s.base + t] = new_state(a, s, v, 8 * e + c, a.U[v * a.S + 8 * e + c], rs, dF[v]);
           }
         }
         __syncthreads();

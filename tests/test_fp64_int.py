@@ -1,7 +1,8 @@
-"""FP64 products on the integer pipes (``csrc/fp64_int.cuh``): the same bits as
-the native product for normal operands with a normal product, on the CPU (the
-header compiled for the host)."""
+"""FP64 arithmetic on the integer pipes (``csrc/fp64_int.cuh``) on the CPU (the
+header compiled for the host): products with the same bits as the native product
+for normal operands with a normal product; sums of six against the exact sum."""
 import ctypes
+import math
 import os
 import subprocess
 
@@ -22,6 +23,14 @@ extern "C" void mul_many(const uint64_t *a, const uint64_t *b, uint64_t *c, long
 }
 extern "C" void mul_many0(const uint64_t *a, const uint64_t *b, uint64_t *c, long n) {
   for (long i = 0; i < n; ++i) c[i] = amr::mul_bits<true>(a[i], b[i]);
+}
+extern "C" void sum_many(const uint64_t *a, uint64_t *c, unsigned char *ok, long n) {
+  for (long i = 0; i < n; ++i) {
+    const uint64_t x[6] = {a[6 * i], a[6 * i + 1], a[6 * i + 2], a[6 * i + 3], a[6 * i + 4], a[6 * i + 5]};
+    bool o;
+    c[i] = amr::sum6_bits<0x2A>(x, o);
+    ok[i] = o;
+  }
 }
 """
 
@@ -84,3 +93,33 @@ def test_products_below_the_normal_range_are_zero(lib):
     lib.mul_many0(_ptr(a), _ptr(b), _ptr(c), ctypes.c_long(n))
     assert ok.sum() > n // 2 and np.count_nonzero(want[ok] == 0) > n // 4
     assert np.array_equal(c[ok], want.view(np.uint64)[ok])
+
+
+@pytest.mark.parametrize("spread", [0, 2, 30, 60, 500])
+def test_sums_of_six_round_once(lib, spread):
+    rng = np.random.default_rng(5 + spread)
+    n = 20000
+    a = _bits(rng, 6 * n, spread).reshape(n, 6)
+    a[::3, 1] = a[::3, 0]                              # differences that cancel
+    a[1::3, 3] = a[1::3, 2] ^ np.uint64(1)             # nearly
+    a[::5, 4:] &= np.uint64(1 << 63)                   # zeros of either sign
+    a[:9] &= np.uint64(1 << 63)
+    x, c, ok = a.view(np.float64), np.zeros(n, np.uint64), np.zeros(n, np.uint8)
+    lib.sum_many(_ptr(a), _ptr(c), _ptr(ok), ctypes.c_long(n))
+    assert ok.all()
+    got = c.view(np.float64)
+    for r, t in zip(got, x * [1, -1, 1, -1, 1, -1]):
+        # five terms lose less than 2^-7 units in the last place of the largest each
+        assert abs(math.fsum([r, *-t])) <= 0.5 * math.ulp(r) + 5 * 2.0 ** -7 * math.ulp(abs(t).max())
+
+
+def test_sums_at_the_ends_of_the_range(lib):
+    a = np.zeros((7, 6))
+    a[0, 2], a[1, 5], a[2, 0] = np.inf, np.nan, 2.0 ** 1020  # refused
+    a[3, 1] = 5e-324                                         # below the normal range: zero
+    a[4, 3], a[5, 2] = 2.0 ** -1022, -(2.0 ** -960)          # exact
+    a[6, :] = 2.0 ** 1018
+    c, ok = np.zeros(7, np.uint64), np.zeros(7, np.uint8)
+    lib.sum_many(_ptr(a), _ptr(c), _ptr(ok), ctypes.c_long(7))
+    assert ok.tolist() == [0, 0, 0, 1, 1, 1, 1]
+    assert c.view(np.float64)[3:].tolist() == [0.0, -(2.0 ** -1022), -(2.0 ** -960), 0.0]

@@ -180,3 +180,23 @@ def test_repack_rejects_bad_arguments_and_keeps_the_handle():
     for q in range(2):
         assert np.array_equal(b.select(q).read(3)[1], before[q])
     b.close()
+
+
+@pytest.mark.parametrize("precision", [8, 4])
+def test_short_and_long_lists_step_alike(precision):
+    """A mesh alone has levels of at most 15 thousand local cells (more threads per
+    cell); 24 copies of it in one batch share lists of some 300 thousand (the
+    kernels that fill the GPU): the same states, reflux and restriction included."""
+    from paper_2607_20704_gb300 import amr
+    pr = inputs.random_mesh(3, 6, seed=5)
+    kw = dict(precision=precision, nsubgrid=0, tile=64, schedule=0)
+    alone = amr.Mesh(*pr.mesh_args(), **pr.params(), **kw)
+    assert alone.advance(3, sync=True) > 0
+    with_copies = amr.Mesh.batch([pr] * 24, **kw)
+    with_copies.advance(3, sync=True)
+    for q in (0, 11, 23):
+        with_copies.select(q)
+        for l in alone.levels():
+            assert np.array_equal(alone.read(l)[1], with_copies.read(l)[1]), (q, l)
+    with_copies.close()
+    alone.close()
