@@ -134,6 +134,8 @@ struct HostPin {
   }
 };
 
+constexpr int kMaxTile = 512;  // cells
+
 // level-step launch domains of a segment
 enum Dom {
   DOM_CELLS = 0, DOM_REAL = 1, DOM_GHOST5 = 2, DOM_UPDATE = 3, DOM_BLOCKS = 4, DOM_COMMIT = 5, DOM_RESTRICT = 6,
@@ -812,6 +814,9 @@ static void run_list(amr_mesh *h, int kid, void (*kern)(StepArgs<T>), StepArgs<T
   if (L.ntile[dom] == 0) return;
   a.tiles = tile_list(h, L, dom);
   int grid = a.tiles.ntiles * per_tile;
+  // beyond the default limit: the largest tile's need, the same from every handle
+  if (smem * h->tile_size > (48 << 10))
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem * kMaxTile));
   if (h->persistent) {
     int per_sm = 0;
     for (auto &o : h->occ)
@@ -895,12 +900,12 @@ static void run_prolong(amr_mesh *h, StepArgs<T> a, const SegList &L, const SegL
 //   FP64  levels of 2-15 thousand cells (random mesh 3-6) 0.308 against 0.333 ms,
 //         a level of 33 thousand 41.1 us both, levels of 25-72 thousand 118 against
 //         111 us (Sod 5-6), one of 262 thousand 162 against 146 us
-//   FP32  random mesh 3-6 0.202 against 0.280 ms, Sod 5-6 53 against 66 us, levels
-//         of 15-100 thousand (Sedov 6-9) 0.234 against 0.310 ms, one of 262
-//         thousand 48.6 against 42.7 us: every face is solved twice there, but
-//         nothing is stored in between
+//   FP32  random mesh 3-6 0.179 against 0.221 ms, levels of 15-50 thousand (Sedov
+//         6-9) 0.212 against 0.257 ms, one of 33 thousand 22.6 against 20.6 us, of
+//         68-73 thousand 0.480 against 0.465 ms (clustered 6-9) and 47 against
+//         49 us (Sod 5-6), of 262 thousand 47.8 against 37.8 us
 template <class T>
-constexpr int kSmallList = sizeof(T) == 8 ? 16384 : 131072;
+constexpr int kSmallList = sizeof(T) == 8 ? 16384 : 65536;
 
 template <class T>
 static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double dt, const SegList **pend) {
@@ -935,9 +940,8 @@ static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double d
   if constexpr (sizeof(T) == 4) {
     run_list(h, K_PREDICT, k_predict_u, a, L, DOM_CELLS);
     if (!small) {
-      // primitives recomputed inside the predictor; each leaf cell solves its six
-      // faces and updates itself
-      run_list(h, K_FLUX, k_flux_update, a, L, DOM_REAL, 20);
+      // primitives recomputed inside the predictor; fluxes stay in the tile
+      run_list(h, K_FLUX, k_flux_update, a, L, DOM_REAL, kFluxSmem);
       if (L.ntile[DOM_REFLUX]) *pend = &L;
       return;
     }

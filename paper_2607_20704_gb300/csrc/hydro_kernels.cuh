@@ -486,15 +486,44 @@ __device__ __forceinline__ void predictor(const SegCtx<double> &s, const double 
     predictor_fp64<MulFp64>(s, w, dw, ws);
 }
 
-template <class T>
-__device__ __forceinline__ void store_q(const StepArgs<T> &a, int o, const T (&ws)[5],
-                                        const T (&dw)[3][5]) {
+// The predictor's results: FP64 as 20 arrays; FP32 as five arrays of four values
+// each (W* without pressure; the pressure and its three slopes; the other slopes per
+// axis), so that a face's side takes three loads instead of ten.
+__device__ __forceinline__ void store_q(const StepArgs<double> &a, int o, const double (&ws)[5],
+                                        const double (&dw)[3][5]) {
 #pragma unroll
   for (int v = 0; v < 5; ++v) a.Q[v * a.LS + o] = ws[v];
 #pragma unroll
   for (int d = 0; d < 3; ++d)
 #pragma unroll
     for (int v = 0; v < 5; ++v) a.Q[(5 + 5 * d + v) * a.LS + o] = dw[d][v];
+}
+__device__ __forceinline__ void store_q(const StepArgs<float> &a, int o, const float (&ws)[5],
+                                        const float (&dw)[3][5]) {
+  float4 *q = reinterpret_cast<float4 *>(a.Q) + o;
+  q[0] = make_float4(ws[0], ws[1], ws[2], ws[3]);
+  q[a.LS] = make_float4(ws[4], dw[0][4], dw[1][4], dw[2][4]);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) q[(2 + d) * a.LS] = make_float4(dw[d][0], dw[d][1], dw[d][2], dw[d][3]);
+}
+// one side of a face normal to axis D: W* + h dW of local cell o (h = 1/2: its plus
+// face, -1/2: its minus face).  Q is read-only while faces are solved
+__device__ __forceinline__ void load_side(const StepArgs<double> &a, int o, int D, double h, double (&q)[5]) {
+  const double *Q = a.Q + o, *S = Q + (5 + 5 * D) * a.LS;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) q[v] = __ldg(Q + v * a.LS) + h * __ldg(S + v * a.LS);
+}
+__device__ __forceinline__ void side_of(const float4 &w, const float4 &p, const float4 &d, int D, float h,
+                                        float (&q)[5]) {
+  q[0] = w.x + h * d.x;
+  q[1] = w.y + h * d.y;
+  q[2] = w.z + h * d.z;
+  q[3] = w.w + h * d.w;
+  q[4] = p.x + h * (D == 0 ? p.y : D == 1 ? p.z : p.w);
+}
+__device__ __forceinline__ void load_side(const StepArgs<float> &a, int o, int D, float h, float (&q)[5]) {
+  const float4 *Q = reinterpret_cast<const float4 *>(a.Q) + o;
+  side_of(__ldg(Q), __ldg(Q + a.LS), __ldg(Q + (2 + D) * a.LS), D, h, q);
 }
 
 // FP64: one thread per cell, an oct in 8 neighbouring lanes.  Along each axis a
@@ -556,24 +585,30 @@ __global__ void k_predict(StepArgs<double> a) {
 // FP32: primitives derived from U directly (no W array): the cell's own and its
 // three outer neighbours' are formed, the three inner ones come from the lanes of
 // its oct (four conversions and 20 gathered loads per cell instead of seven
-// and 35)
-__global__ void __launch_bounds__(512, 3) k_predict_u(StepArgs<float> a) {
+// and 35).  128^3 uniform 48 us (53 at 40 registers with the neighbours one after the
+// other), of which 31 are its 100 bytes per cell.
+__global__ void __launch_bounds__(512, 2) k_predict_u(StepArgs<float> a) {
   warp_tile_loop(a, [&](const SegCtx<float> &s, int t) {  // tiles start at multiples of 8: octs are whole
     const bool on = t < 8 * (s.nl + s.ncl);
     const unsigned lanes = __ballot_sync(0xFFFFFFFFu, on);
     if (!on) return;
     const int e = ext_of_local(a, s, t >> 3);
     const int c = t & 7;
+    // the three outer neighbours, or the cell itself (outer ring of a ghost oct, slopes
+    // never used): all addresses before the first wait
+    int out[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int to = nbr_local(a, s, t, e, c, d, (c >> d) & 1);
+      out[d] = to >= 0 ? to : t;
+    }
     float w[5], dw[3][5], ws[5];
     prim_at(a, s, t, w);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const bool up = (c >> d) & 1;  // the pair's cell on the plus side
-      const int to = nbr_local(a, s, t, e, c, d, up ? 1 : 0);
       float wo[5];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) wo[v] = w[v];  // outer ring of a ghost oct (slopes 0): never used
-      if (to >= 0) prim_at(a, s, to, wo);
+      prim_at(a, s, out[d], wo);
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         const float wi = __shfl_xor_sync(lanes, w[v], 1 << d);
@@ -726,14 +761,8 @@ template <class T>
 __device__ __forceinline__ void face_flux(const StepArgs<T> &a, const SegCtx<T> &s, int D, int tl, int tr,
                                           T (&F)[5]) {
   T qL[5], qR[5];
-  const T *Ql = a.Q + (s.base + tl), *Qr = a.Q + (s.base + tr);
-  const int64_t sl = (5 + 5 * D) * a.LS;  // the axis' slopes
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    // Q is read-only while faces are solved
-    qL[v] = __ldg(Ql + v * a.LS) + T(0.5) * __ldg(Ql + sl + v * a.LS);
-    qR[v] = __ldg(Qr + v * a.LS) - T(0.5) * __ldg(Qr + sl + v * a.LS);
-  }
+  load_side(a, s.base + tl, D, T(0.5), qL);
+  load_side(a, s.base + tr, D, T(-0.5), qR);
   face_flux_states(D, s, qL, qR, F);
 }
 
@@ -919,75 +948,123 @@ __global__ void k_update_small(StepArgs<T> a) {
   }
 }
 
-// FP32: the two faces of local cell t along axis D, du = F(minus) - F(plus);
-// each interior face is solved by both of its cells (bit-identically), and a
-// coarse-fine face by its real cell, which also fills the reflux slot
-template <int D>
-__device__ __forceinline__ void faces_dir(const StepArgs<float> &a, const SegCtx<float> &s, int t, int e, int c,
-                                          float (&du)[5]) {
-  float Fm[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, Fp[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  const int tm = nbr_local(a, s, t, e, c, D, 0);
-  if (!cell_is_split(a, s, tm)) {
-    face_flux(a, s, D, tm, t, Fm);
-    if (a.reflux && (tm >> 3) >= s.nl) {
-      const int64_t gslot = reflux_slot(D, s.clo, s.nl, tm >> 3, 2 * D + 1, c);
-#pragma unroll
-      for (int v = 0; v < 5; ++v)
-        a.C[v * a.CS + checked(gslot, 0, a.CS, a.err)] = (-1.0f * s.dtdx) * Fm[v] / 8.0f;
-    }
-  }
-  const int tp = nbr_local(a, s, t, e, c, D, 1);
-  if (!cell_is_split(a, s, tp)) {
-    face_flux(a, s, D, t, tp, Fp);
-    if (a.reflux && (tp >> 3) >= s.nl) {
-      const int64_t gslot = reflux_slot(D, s.clo, s.nl, tp >> 3, 2 * D, c);
-#pragma unroll
-      for (int v = 0; v < 5; ++v)
-        a.C[v * a.CS + checked(gslot, 0, a.CS, a.err)] = (1.0f * s.dtdx) * Fp[v] / 8.0f;
-    }
-  }
-#pragma unroll
-  for (int v = 0; v < 5; ++v) du[v] = Fm[v] - Fp[v];
-}
-
-// FP32 flux and update, thread per cell: six faces, the update and the
-// restriction of the warp's octs.  (Three threads per cell, one per axis, meeting
-// in shared memory, spill nothing but took 474 instead of 395 us per Sedov coarse
-// step: the axes no longer share the cell's state, and two thirds of the threads
-// wait out the update.)  domain: 8 nl
+// FP32 flux and update, thread per cell of a tile.  Each leaf cell solves its plus
+// faces into shared memory; a minus face belongs to the cell beyond it, and only
+// where that one lies outside the tile (at most 12 of an oct's faces) it goes to a
+// list that the block solves next, without idle lanes.  A tile of 512 cells of a
+// refined region, 8^3 in Hilbert order, solves 3.4 faces per cell instead of both
+// cells of a face solving it, and stores no flux.  Then the update and the
+// restriction of the warp's octs.  Bound by the latency of its gathered loads: the
+// neighbours' indices are all loaded before the first is needed.  128^3 uniform, us:
+// six solves per cell from 20 predictor arrays 136; plus faces shared 123; with
+// four-value arrays and indices first 100 (256^3: 896 -> 706; Sedov 7-10 per coarse
+// step 427 -> 365); at 62 registers 120, at 32 with spills 140.  domain: 8 nl
+constexpr int kFluxSmem = 15 * 4 + 5 * 6 + 2 * 6 + 2;  // bytes per thread
 __global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<float> a) {
-  extern __shared__ float flux_smem[];  // the block's new states [5][threads]
-  const int lane = threadIdx.x & 31;
-  warp_tile_loop(a, [&](const SegCtx<float> &s, int t) {
-    if (t < 8 * s.nl) {
-      const int e = s.lo + (t >> 3), c = t & 7, g = 8 * e + c;
-      float u[5];
-      if (cell_is_split(a, s, t)) {
+  extern __shared__ float flux_smem[];
+  const int nth = blockDim.x, cap = nth + nth / 2, tid = threadIdx.x, lane = tid & 31;
+  float *plus = flux_smem, *minus = plus + 15 * nth;  // fluxes [3][5][nth], [5][cap]
+  int *cell = reinterpret_cast<int *>(minus + 5 * cap), *beyond = cell + cap;  // [cap]: axis, thread; minus cell
+  int *listed = beyond + cap;
+  warp_tile_loop(a, [&](const SegCtx<float> &s, int t) {  // the same tile for the whole block
+    if (tid == 0) *listed = 0;
+    __syncthreads();
+    const int t0 = t - tid, e = s.lo + (t >> 3), c = t & 7, g = 8 * e + c;
+    const uint32_t split = t < 8 * s.nl ? __ldg(a.son + e) : ~0u;  // of the oct's cells
+    const bool leaf = !((split >> c) & 1u);
+    // the neighbour in the next oct along each axis, or -1 where that is split (the
+    // other neighbour is in this oct)
+    int out[3] = {-1, -1, -1};
+    if (leaf) {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + g];
-      } else {
-        float dx[5], dy[5], dz[5];
-        faces_dir<0>(a, s, t, e, c, dx);
-        faces_dir<1>(a, s, t, e, c, dy);
-        faces_dir<2>(a, s, t, e, c, dz);
-        const int rs = reflux_of(a, g);
+      for (int D = 0; D < 3; ++D) out[D] = nbr_local(a, s, t, e, c, D, (c >> D) & 1);
 #pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          u[v] = new_state(a, s, v, g, a.U[v * a.S + g], rs, (dx[v] + dy[v]) + dz[v]);
-          a.U[v * a.S + g] = u[v];
+      for (int D = 0; D < 3; ++D)
+        if (out[D] >= 0 && cell_is_split(a, s, out[D])) out[D] = -1;
+    }
+    int from[3];  // of a minus face's flux: a thread's plus face, -2 - place in the list, or -1 (none)
+#pragma unroll
+    for (int D = 0; D < 3; ++D) {
+      const bool up = (c >> D) & 1;
+      const bool outside = leaf && !up && out[D] >= 0 && (out[D] < t0 || out[D] >= t0 + nth || (out[D] >> 3) >= s.nl);
+      from[D] = up ? ((split >> (c ^ (1 << D))) & 1u ? -1 : tid ^ (1 << D)) : out[D] < 0 ? -1 : out[D] - t0;
+      const unsigned add = __ballot_sync(0xFFFFFFFFu, outside);
+      if (add) {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(listed, __popc(add));
+        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(add & ((1u << lane) - 1u));
+        if (outside) {
+          cell[at] = D << 16 | tid;
+          beyond[at] = out[D];
+          from[D] = -2 - at;
         }
       }
-      if (s.flags & kSegRestrict) {
+    }
+    if (leaf) {
+      const float4 *Q = reinterpret_cast<const float4 *>(a.Q) + s.base + t;
+      const float4 w = __ldg(Q), p = __ldg(Q + a.LS);
 #pragma unroll
-        for (int v = 0; v < 5; ++v) flux_smem[v * blockDim.x + threadIdx.x] = u[v];
+      for (int D = 0; D < 3; ++D) {
+        const bool up = (c >> D) & 1;
+        const int tp = up ? out[D] : (split >> (c ^ (1 << D))) & 1u ? -1 : t ^ (1 << D);
+        float F[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        if (tp >= 0) {
+          float qL[5], qR[5];
+          side_of(w, p, __ldg(Q + (2 + D) * a.LS), D, 0.5f, qL);
+          load_side(a, s.base + tp, D, -0.5f, qR);
+          face_flux_states(D, s, qL, qR, F);
+          if (a.reflux && (tp >> 3) >= s.nl) {
+            const int64_t gslot = reflux_slot(D, s.clo, s.nl, tp >> 3, 2 * D, c);
+#pragma unroll
+            for (int v = 0; v < 5; ++v)
+              a.C[v * a.CS + checked(gslot, 0, a.CS, a.err)] = (1.0f * s.dtdx) * F[v] / 8.0f;
+          }
+        }
+#pragma unroll
+        for (int v = 0; v < 5; ++v) plus[(5 * D + v) * nth + tid] = F[v];
       }
     }
+    __syncthreads();
+    for (int i = tid; i < *listed; i += nth) {
+      const int D = cell[i] >> 16, tc = t0 + (cell[i] & 0xFFFF), tb = beyond[i];
+      float F[5];
+      face_flux(a, s, D, tb, tc, F);
+      if (a.reflux && (tb >> 3) >= s.nl) {
+        const int64_t gslot = reflux_slot(D, s.clo, s.nl, tb >> 3, 2 * D + 1, tc & 7);
+#pragma unroll
+        for (int v = 0; v < 5; ++v)
+          a.C[v * a.CS + checked(gslot, 0, a.CS, a.err)] = (-1.0f * s.dtdx) * F[v] / 8.0f;
+      }
+#pragma unroll
+      for (int v = 0; v < 5; ++v) minus[v * cap + i] = F[v];
+    }
+    __syncthreads();
+    float u[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    if (t < 8 * s.nl) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + g];
+    }
+    if (leaf) {
+      const int rs = reflux_of(a, g);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        float m[3], p[3];
+#pragma unroll
+        for (int D = 0; D < 3; ++D) {
+          p[D] = plus[(5 * D + v) * nth + tid];
+          m[D] = from[D] >= 0 ? plus[(5 * D + v) * nth + from[D]] : from[D] == -1 ? 0.0f : minus[v * cap - 2 - from[D]];
+        }
+        u[v] = new_state(a, s, v, g, u[v], rs, flux_sum(m[0], p[0], m[1], p[1], m[2], p[2]));
+        a.U[v * a.S + g] = u[v];
+      }
+    }
+    __syncthreads();  // the fluxes are read
     if (s.flags & kSegRestrict) {  // the warp's octs, a lane per (oct, variable)
+#pragma unroll
+      for (int v = 0; v < 5; ++v) plus[v * nth + tid] = u[v];
       __syncwarp();
       const int q = ((t - lane) >> 3) + (lane & 3), v = lane >> 2;
-      if (v < 5 && q < s.nl)
-        restrict_oct(a, s, q, v, flux_smem + v * blockDim.x + (threadIdx.x - lane) + 8 * (lane & 3));
-      __syncwarp();
+      if (v < 5 && q < s.nl) restrict_oct(a, s, q, v, plus + v * nth + (tid - lane) + 8 * (lane & 3));
     }
   });
 }

@@ -182,14 +182,14 @@ def test_repack_rejects_bad_arguments_and_keeps_the_handle():
     b.close()
 
 
-@pytest.mark.parametrize("precision", [8, 4])
-def test_short_and_long_lists_step_alike(precision):
+@pytest.mark.parametrize("precision,tile", [(8, 64), (4, 64), (4, 512)])
+def test_short_and_long_lists_step_alike(precision, tile):
     """A mesh alone has levels of at most 15 thousand local cells (more threads per
     cell); 24 copies of it in one batch share lists of some 300 thousand (the
     kernels that fill the GPU): the same states, reflux and restriction included."""
     from paper_2607_20704_gb300 import amr
     pr = inputs.random_mesh(3, 6, seed=5)
-    kw = dict(precision=precision, nsubgrid=0, tile=64, schedule=0)
+    kw = dict(precision=precision, nsubgrid=0, tile=tile, schedule=0)
     alone = amr.Mesh(*pr.mesh_args(), **pr.params(), **kw)
     assert alone.advance(3, sync=True) > 0
     with_copies = amr.Mesh.batch([pr] * 24, **kw)
