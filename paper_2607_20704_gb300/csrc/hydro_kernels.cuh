@@ -827,15 +827,20 @@ __device__ __forceinline__ float flux_sum(float xm, float xp, float ym, float yp
   return ((xm - xp) + (ym - yp)) + (zm - zp);
 }
 
-// new state (u + dt/dx dF) + R of variable v of leaf cell g, dF its flux sum, rs
-// the slot of its pending reflux R (or -1); R <- 0
+// variable v of the pending reflux R in slot rs (-1: none).  Loaded with the fluxes,
+// before their sum: after it the load's latency comes on top (clustered 6-9, update
+// per coarse step: 439 instead of 253 us)
 template <class T>
-__device__ __forceinline__ T new_state(const StepArgs<T> &a, const SegCtx<T> &s, int v, int g, T u, int rs, T dF) {
+__device__ __forceinline__ T pending(const StepArgs<T> &a, int v, int rs) {
+  return rs >= 0 ? a.Rc[v * int64_t(a.NC) + rs] : T(0);
+}
+// new state (u + dt/dx dF) + R of variable v, dF its flux sum; R <- 0
+template <class T>
+__device__ __forceinline__ T new_state(const StepArgs<T> &a, const SegCtx<T> &s, int v, T u, int rs, T r, T dF) {
   u = u + s.dtdx * dF;
   if (rs >= 0) {
-    T *Rv = a.Rc + v * int64_t(a.NC) + rs;
-    u = u + *Rv;
-    *Rv = T(0);
+    u = u + r;
+    a.Rc[v * int64_t(a.NC) + rs] = T(0);
   }
   return u;
 }
@@ -868,10 +873,9 @@ __device__ __forceinline__ void restrict_oct(const StepArgs<T> &a, const SegCtx<
 // the pending reflux of its leaf cells.
 
 // FP64, a list that fills the GPU: a thread per cell, one variable after the other.
-// Sedov 7-10 / clustered 6-9, us per coarse step: 458 / 275; the sums on the FP64
-// pipe 481 / 385; all five variables unrolled 455 / 367; a thread per (cell,
-// variable) 672 / 463 (the cell's five index loads are repeated).  A branch around
-// the sum for warps of gas at rest: 441 / 441.
+// Sedov 7-10 / clustered 6-9, us per coarse step: 359 / 253; the sums on the FP64
+// pipe 481 / 385, the bound of that form.  The loads of the next variable ahead of
+// the sum: 371 / 256; at 40 registers 369 / 269.
 // domain: 8 nl, + 5 ncl (if kSegReflux)
 __global__ void __launch_bounds__(512, 2) k_update(StepArgs<double> a) {
   extern __shared__ double update_smem[];  // the block's new states [5][threads]
@@ -892,7 +896,9 @@ __global__ void __launch_bounds__(512, 2) k_update(StepArgs<double> a) {
         double u = a.U[v * a.S + g];
         if (leaf) {
           const double *Fx = a.F + v * a.LS + s.base, *Fy = Fx + 5 * a.LS, *Fz = Fy + 5 * a.LS;
-          u = new_state(a, s, v, g, u, rs, flux_sum(Fx[mx], Fx[t], Fy[my], Fy[t], Fz[mz], Fz[t]));
+          const double xm = Fx[mx], xp = Fx[t], ym = Fy[my], yp = Fy[t], zm = Fz[mz], zp = Fz[t];
+          const double r = pending(a, v, rs);
+          u = new_state(a, s, v, u, rs, r, flux_sum(xm, xp, ym, yp, zm, zp));
           a.U[v * a.S + g] = u;
         }
         if (s.flags & kSegRestrict) update_smem[v * blockDim.x + threadIdx.x] = u;
@@ -932,7 +938,9 @@ __global__ void k_update_small(StepArgs<T> a) {
         const T *Fx = a.F + v * a.LS + s.base, *Fy = Fx + 5 * a.LS, *Fz = Fy + 5 * a.LS;
         const int mx = nbr_local(a, s, t, e, c, 0, 0), my = nbr_local(a, s, t, e, c, 1, 0),
                   mz = nbr_local(a, s, t, e, c, 2, 0);
-        u = new_state(a, s, v, g, u, reflux_of(a, g), flux_sum(Fx[mx], Fx[t], Fy[my], Fy[t], Fz[mz], Fz[t]));
+        const int rs = reflux_of(a, g);
+        const T xm = Fx[mx], xp = Fx[t], ym = Fy[my], yp = Fy[t], zm = Fz[mz], zp = Fz[t], r = pending(a, v, rs);
+        u = new_state(a, s, v, u, rs, r, flux_sum(xm, xp, ym, yp, zm, zp));
         a.U[v * a.S + g] = u;
       }
       sm[threadIdx.x] = u;
@@ -1054,7 +1062,7 @@ __global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<float> a) {
           p[D] = plus[(5 * D + v) * nth + tid];
           m[D] = from[D] >= 0 ? plus[(5 * D + v) * nth + from[D]] : from[D] == -1 ? 0.0f : minus[v * cap - 2 - from[D]];
         }
-        u[v] = new_state(a, s, v, g, u[v], rs, flux_sum(m[0], p[0], m[1], p[1], m[2], p[2]));
+        u[v] = new_state(a, s, v, u[v], rs, pending(a, v, rs), flux_sum(m[0], p[0], m[1], p[1], m[2], p[2]));
         a.U[v * a.S + g] = u[v];
       }
     }

@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(Rock<NS>::THREADS, Rock<NS>::template min_bloc
         const T *Fv = sF + v * FS;
         const T dF = flux_sum(Fv[gi], Fv[pf[0]], Fv[5 * FS + gi], Fv[5 * FS + pf[1]], Fv[10 * FS + gi],
                               Fv[10 * FS + pf[2]]);
-        out[v * a.LS] = new_state(a, s, v, g, __ldg(a.U + v * a.S + g), rs, dF);
+        out[v * a.LS] = new_state(a, s, v, __ldg(a.U + v * a.S + g), rs, pending(a, v, rs), dF);
       }
     }
     __syncthreads();
@@ -667,7 +667,8 @@ __global__ void __launch_bounds__(Sweep<NS>::THREADS) k_sweep(StepArgs<T> a, con
             const int rs = reflux_of(a, 8 * e + c);
 #pragma unroll
             for (int v = 0; v < 5; ++v)  // into the scratch: other blocks may still read the old state
-              a.W[v * int64_t(a.LS) + s.base + t] = new_state(a, s, v, 8 * e + c, a.U[v * a.S + 8 * e + c], rs, dF[v]);
+              a.W[v * int64_t(a.LS) + s.base + t] =
+                  new_state(a, s, v, a.U[v * a.S + 8 * e + c], rs, pending(a, v, rs), dF[v]);
           }
         }
         __syncthreads();
