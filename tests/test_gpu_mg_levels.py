@@ -209,3 +209,24 @@ def test_errors_and_regrid():
     else:
         assert np.array_equal(g.read_phi_level(g.levelmin), before)
     g.close()
+
+
+def test_repeated_calls_replay_the_same_solve():
+    """Calls without residuals are recorded and replayed: the same potentials as
+    direct launches while the density, the arguments and the entry point change."""
+    from paper_2607_20704_gb300 import amr
+    pr = _meshes()[1]
+    a, b = (amr.Mesh(*pr.mesh_args(), **pr.params(), use_graphs=g) for g in (True, False))
+    for call in (3, 3, 3, -2, -2, -2, 3, 2, 2, 2):  # cycles; negative: the base level only
+        for m in (a, b):
+            if call < 0:
+                m.poisson(1.5, -call, residuals=False)
+            else:
+                m.poisson_levels(1.0, call, residuals=False)
+        assert np.array_equal(a.read_phi(), b.read_phi())
+        for l in a.levels() if call > 0 else ():
+            assert np.array_equal(a.read_phi_level(l), b.read_phi_level(l)), (call, l)
+        a.advance(1, sync=True)
+        b.advance(1, sync=True)
+    a.close()
+    b.close()

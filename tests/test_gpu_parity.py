@@ -88,6 +88,26 @@ def test_cfl_dt_matches(seed):
     assert abs(g.cfl_dt() - o.cfl_dt()) <= 1e-14 * o.cfl_dt()
 
 
+@pytest.mark.parametrize("cells", [
+    dict(E=1.0 + 1e-12), dict(E=1e25), dict(rho=1e-30), dict(rho=1e25, E=3.0), dict(mom=1e-200, E=2.0), dict(mom=1.4),
+    dict(mom=1e12, E=1e25), dict(E=1e-40), dict(E=1.0)])
+def test_cfl_finds_one_cell_among_equals(cells):
+    """The FP64 time step screens cells by an FP32 bound: one cell that differs from
+    all others by less than that bound resolves, or lies outside its range."""
+    prob = _random(1, 3, 5)
+    g, o = pair(prob)
+    for l in o.levels():
+        n = 8 * o.num_octs(l)
+        U = np.zeros((5, n))
+        U[0], U[1], U[4] = 1.0, 0.1, 1.0
+        if l == prob.levelmax:
+            c = n // 2 + 3
+            U[0, c], U[2, c], U[4, c] = cells.get("rho", 1.0), cells.get("mom", 0.0), cells.get("E", 1.0)
+        g.write(l, U)
+        o.write(l, U)
+    assert abs(g.cfl_dt() - o.cfl_dt()) <= 1e-14 * o.cfl_dt()
+
+
 @pytest.mark.parametrize("seed", SEEDS)
 def test_each_level_step_matches(seed):
     prob = _random(seed, 3, 6)
