@@ -893,19 +893,14 @@ static void run_prolong(amr_mesh *h, StepArgs<T> a, const SegList &L, const SegL
   launch(h, K_PROLONG, k_prolong<T>, dim3(unsigned(grid)), dim3(unsigned(h->tile_size)), a, p);
 }
 
-// Up to this many local cells a list does not fill the GPU, and a level step lasts
-// as long as its kernels' chains of loads and arithmetic: it takes the kernels with
-// more threads and less per thread, k_update_small and, in FP32, a solve per face
-// (k_flux).  Times of a step, these kernels against the others:
-//   FP64  levels of 2-15 thousand cells (random mesh 3-6) 0.308 against 0.333 ms,
-//         a level of 33 thousand 41.1 us both, levels of 25-72 thousand 118 against
-//         111 us (Sod 5-6), one of 262 thousand 162 against 146 us
-//   FP32  random mesh 3-6 0.179 against 0.221 ms, levels of 15-50 thousand (Sedov
-//         6-9) 0.212 against 0.257 ms, one of 33 thousand 22.6 against 20.6 us, of
-//         68-73 thousand 0.480 against 0.465 ms (clustered 6-9) and 47 against
-//         49 us (Sod 5-6), of 262 thousand 47.8 against 37.8 us
-template <class T>
-constexpr int kSmallList = sizeof(T) == 8 ? 16384 : 65536;
+// FP64: up to this many local cells a list does not fill the GPU, and the update
+// lasts as long as its chain of loads and arithmetic: it takes k_update_small, with a
+// thread per (cell, variable).  Times of a step, that kernel against the other: levels
+// of 2-15 thousand cells (random mesh 3-6) 0.295 against 0.334 ms, of 15-50 thousand
+// (Sedov 6-9) 0.486 against 0.511 ms, of 25-72 thousand (Sod 5-6) 107 against 109 us;
+// with lists of up to 131 thousand in it, clustered 6-9, 1.136 against 1.125 ms; a
+// level of 262 thousand 162 against 140 us.
+constexpr int kSmallList = 65536;
 
 template <class T>
 static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double dt, const SegList **pend) {
@@ -936,28 +931,25 @@ static void run_segments(amr_mesh *h, const SegList &L, bool device_dt, double d
     run_list(h, K_COMMIT, k_commit_post<T>, a, L, DOM_COMMIT);
     return;
   }
-  const bool small = L.ls <= kSmallList<T>;
   if constexpr (sizeof(T) == 4) {
+    // primitives recomputed inside the predictor; fluxes stay in the tile
     run_list(h, K_PREDICT, k_predict_u, a, L, DOM_CELLS);
-    if (!small) {
-      // primitives recomputed inside the predictor; fluxes stay in the tile
-      run_list(h, K_FLUX, k_flux_update, a, L, DOM_REAL, kFluxSmem);
-      if (L.ntile[DOM_REFLUX]) *pend = &L;
-      return;
-    }
+    const auto kern = h->tile_size == 64    ? k_flux_update<64>
+                      : h->tile_size == 128 ? k_flux_update<128>
+                      : h->tile_size == 256 ? k_flux_update<256>
+                                            : k_flux_update<512>;
+    run_list(h, K_FLUX, kern, a, L, DOM_REAL, kFluxSmem);
+    if (L.ntile[DOM_REFLUX]) *pend = &L;
   } else {
-    // FP64: every predictor and every face solve exactly once
+    // every predictor and every face solve exactly once
     run_list(h, K_PRIM, k_ghost_prim, a, L, DOM_CELLS, 16);
     run_list(h, K_PREDICT, k_predict, a, L, DOM_CELLS);
-  }
-  run_list(h, K_FLUX, k_flux<T>, a, L, DOM_CELLS, 0, 3);
-  if constexpr (sizeof(T) == 8) {
-    if (!small) {
+    run_list(h, K_FLUX, k_flux, a, L, DOM_CELLS, 0, 3);
+    if (L.ls <= kSmallList)
+      run_list(h, K_UPDATE, k_update_small, a, L, DOM_UPDATE1, 8, 5);
+    else
       run_list(h, K_UPDATE, k_update, a, L, DOM_UPDATE, 40);
-      return;
-    }
   }
-  run_list(h, K_UPDATE, k_update_small<T>, a, L, DOM_UPDATE1, sizeof(T), 5);
 }
 
 // One level step of a list.  *pend: a list whose reflux sums are still to be

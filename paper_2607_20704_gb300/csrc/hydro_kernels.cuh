@@ -783,18 +783,17 @@ __device__ __forceinline__ int64_t reflux_slot(int D, int clo, int nl, int gq, i
 // axes are consecutive blocks: the faces of a small level are solved at once
 // (one after the other they are a chain of three solves, which bounds a level
 // that does not fill the GPU), and a large level finds the cells' states in L2.
-template <class T>
-__global__ void k_flux(StepArgs<T> a) {
+__global__ void k_flux(StepArgs<double> a) {
   for (int tb = blockIdx.x; tb < 3 * a.tiles.ntiles; tb += gridDim.x) {
     const int ti = tb / 3, D = tb - 3 * ti;
     const Tile td = tile_at(a.tiles, ti);
-    SegCtx<T> s;
+    SegCtx<double> s;
     if (!open_segment(a, td.seg, s)) continue;
     const int t = td.start + threadIdx.x;
     if (t >= 8 * (s.nl + s.ncl)) continue;
     const int q = t >> 3, c = t & 7;
     const bool real = q < s.nl;
-    T F[5] = {T(0), T(0), T(0), T(0), T(0)};
+    double F[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     const int tn = nbr_local(a, s, t, ext_of_local(a, s, q), c, D, 1);
     if (tn >= 0) {
       const bool nreal = (tn >> 3) < s.nl;
@@ -805,10 +804,10 @@ __global__ void k_flux(StepArgs<T> a) {
           // ghost on the minus side: its plus face (sigma -1)
           const int64_t gslot = real ? reflux_slot(D, s.clo, s.nl, tn >> 3, 2 * D, c)
                                      : reflux_slot(D, s.clo, s.nl, t >> 3, 2 * D + 1, c);
-          const T sg8 = real ? T(1) : T(-1);
+          const double sg8 = real ? 1.0 : -1.0;
 #pragma unroll
           for (int v = 0; v < 5; ++v)
-            a.C[v * a.CS + checked(gslot, 0, a.CS, a.err)] = (sg8 * s.dtdx) * F[v] / T(8);
+            a.C[v * a.CS + checked(gslot, 0, a.CS, a.err)] = (sg8 * s.dtdx) * F[v] / 8.0;
         }
       }
     }
@@ -917,29 +916,28 @@ __global__ void __launch_bounds__(512, 2) k_update(StepArgs<double> a) {
   });
 }
 
-// A small list: a thread per (cell, variable), a tile's five variables in
+// FP64, a short list: a thread per (cell, variable), a tile's five variables in
 // consecutive blocks (five times the threads and a fifth of the chain).
 // domain: 8 nl, + ncl (if kSegReflux)
-template <class T>
-__global__ void k_update_small(StepArgs<T> a) {
-  extern __shared__ __align__(8) unsigned char update_bytes[];
-  T *sm = reinterpret_cast<T *>(update_bytes);  // the block's new states
+__global__ void k_update_small(StepArgs<double> a) {
+  extern __shared__ double update_smem[];  // the block's new states
+  double *sm = update_smem;
   const int lane = threadIdx.x & 31;
   for (int tb = blockIdx.x; tb < 5 * a.tiles.ntiles; tb += gridDim.x) {
     const int ti = tb / 5, v = tb - 5 * ti;
     const Tile td = tile_at(a.tiles, ti);
-    SegCtx<T> s;
+    SegCtx<double> s;
     if (!open_segment(a, td.seg, s)) continue;
     const int t = td.start + threadIdx.x;
     if (t < 8 * s.nl) {
       const int e = s.lo + (t >> 3), c = t & 7, g = 8 * e + c;
-      T u = a.U[v * a.S + g];
+      double u = a.U[v * a.S + g];
       if (!cell_is_split(a, s, t)) {
-        const T *Fx = a.F + v * a.LS + s.base, *Fy = Fx + 5 * a.LS, *Fz = Fy + 5 * a.LS;
+        const double *Fx = a.F + v * a.LS + s.base, *Fy = Fx + 5 * a.LS, *Fz = Fy + 5 * a.LS;
         const int mx = nbr_local(a, s, t, e, c, 0, 0), my = nbr_local(a, s, t, e, c, 1, 0),
                   mz = nbr_local(a, s, t, e, c, 2, 0);
         const int rs = reflux_of(a, g);
-        const T xm = Fx[mx], xp = Fx[t], ym = Fy[my], yp = Fy[t], zm = Fz[mz], zp = Fz[t], r = pending(a, v, rs);
+        const double xm = Fx[mx], xp = Fx[t], ym = Fy[my], yp = Fy[t], zm = Fz[mz], zp = Fz[t], r = pending(a, v, rs);
         u = new_state(a, s, v, u, rs, r, flux_sum(xm, xp, ym, yp, zm, zp));
         a.U[v * a.S + g] = u;
       }
@@ -962,18 +960,26 @@ __global__ void k_update_small(StepArgs<T> a) {
 // list that the block solves next, without idle lanes.  A tile of 512 cells of a
 // refined region, 8^3 in Hilbert order, solves 3.4 faces per cell instead of both
 // cells of a face solving it, and stores no flux.  Then the update and the
-// restriction of the warp's octs.  Bound by the latency of its gathered loads: the
-// neighbours' indices are all loaded before the first is needed.  128^3 uniform, us:
-// six solves per cell from 20 predictor arrays 136; plus faces shared 123; with
-// four-value arrays and indices first 100 (256^3: 896 -> 706; Sedov 7-10 per coarse
-// step 427 -> 365); at 62 registers 120, at 32 with spills 140.  domain: 8 nl
-constexpr int kFluxSmem = 15 * 4 + 5 * 6 + 2 * 6 + 2;  // bytes per thread
-__global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<float> a) {
+// restriction of the warp's octs.  Bound by instructions (issue 73 %) and the latency
+// of gathered loads: the neighbours' indices are all loaded before the first is
+// needed, and the state and its pending reflux before the first store, which the
+// compiler would keep them behind.  us, 128^3 uniform / Sedov 7-10 / clustered 6-9 per
+// coarse step: six solves per cell from 20 predictor arrays 136 / 427 / 338; plus
+// faces shared 123 / 415; with four-value arrays and indices first 100 / 365 / 328;
+// loads before stores and the tile size a constant 94 / 288 / 205.  At 62 registers
+// 120, at 32 with spills 140.  A solve per face into memory and an update of its own,
+// with more threads per cell, is no faster on short lists either (random mesh 3-6
+// 0.191 against 0.190 ms, levels of 25-72 thousand cells 51 against 47 us).
+// domain: 8 nl
+constexpr int kFluxSmem = 15 * 4 + 10 * 4 + 2 * 6 + 2;  // bytes per thread
+template <int TH>
+__global__ void __launch_bounds__(TH, 1536 / TH) k_flux_update(StepArgs<float> a) {
   extern __shared__ float flux_smem[];
-  const int nth = blockDim.x, cap = nth + nth / 2, tid = threadIdx.x, lane = tid & 31;
-  float *plus = flux_smem, *minus = plus + 15 * nth;  // fluxes [3][5][nth], [5][cap]
-  int *cell = reinterpret_cast<int *>(minus + 5 * cap), *beyond = cell + cap;  // [cap]: axis, thread; minus cell
-  int *listed = beyond + cap;
+  // fluxes [5][TH]: plus faces along each axis, two halves of the list (at most 1.5 TH)
+  float *const flux = flux_smem;
+  int *const cell = reinterpret_cast<int *>(flux + 25 * TH), *const beyond = cell + TH + TH / 2;
+  int *const listed = beyond + TH + TH / 2;  // list: axis and thread; the cell beyond
+  const int tid = threadIdx.x, lane = tid & 31;
   warp_tile_loop(a, [&](const SegCtx<float> &s, int t) {  // the same tile for the whole block
     if (tid == 0) *listed = 0;
     __syncthreads();
@@ -990,12 +996,14 @@ __global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<float> a) {
       for (int D = 0; D < 3; ++D)
         if (out[D] >= 0 && cell_is_split(a, s, out[D])) out[D] = -1;
     }
-    int from[3];  // of a minus face's flux: a thread's plus face, -2 - place in the list, or -1 (none)
+    int from[3];  // first of the five values of each minus face's flux, -1: none
 #pragma unroll
     for (int D = 0; D < 3; ++D) {
       const bool up = (c >> D) & 1;
-      const bool outside = leaf && !up && out[D] >= 0 && (out[D] < t0 || out[D] >= t0 + nth || (out[D] >> 3) >= s.nl);
-      from[D] = up ? ((split >> (c ^ (1 << D))) & 1u ? -1 : tid ^ (1 << D)) : out[D] < 0 ? -1 : out[D] - t0;
+      const int rel = up ? tid ^ (1 << D) : out[D] - t0;
+      const bool none = up ? (split >> (c ^ (1 << D))) & 1u : out[D] < 0;
+      from[D] = none ? -1 : 5 * D * TH + rel;
+      const bool outside = leaf && !up && !none && (unsigned(rel) >= TH || (out[D] >> 3) >= s.nl);
       const unsigned add = __ballot_sync(0xFFFFFFFFu, outside);
       if (add) {
         int at = 0;
@@ -1004,7 +1012,7 @@ __global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<float> a) {
         if (outside) {
           cell[at] = D << 16 | tid;
           beyond[at] = out[D];
-          from[D] = -2 - at;
+          from[D] = 15 * TH + at + (at >= TH ? 4 * TH : 0);
         }
       }
     }
@@ -1029,11 +1037,11 @@ __global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<float> a) {
           }
         }
 #pragma unroll
-        for (int v = 0; v < 5; ++v) plus[(5 * D + v) * nth + tid] = F[v];
+        for (int v = 0; v < 5; ++v) flux[(5 * D + v) * TH + tid] = F[v];
       }
     }
     __syncthreads();
-    for (int i = tid; i < *listed; i += nth) {
+    for (int i = tid; i < *listed; i += TH) {
       const int D = cell[i] >> 16, tc = t0 + (cell[i] & 0xFFFF), tb = beyond[i];
       float F[5];
       face_flux(a, s, D, tb, tc, F);
@@ -1043,36 +1051,38 @@ __global__ void __launch_bounds__(512, 3) k_flux_update(StepArgs<float> a) {
         for (int v = 0; v < 5; ++v)
           a.C[v * a.CS + checked(gslot, 0, a.CS, a.err)] = (-1.0f * s.dtdx) * F[v] / 8.0f;
       }
+      float *m = flux + 15 * TH + i + (i >= TH ? 4 * TH : 0);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) minus[v * cap + i] = F[v];
+      for (int v = 0; v < 5; ++v) m[v * TH] = F[v];
     }
+    const int rs = leaf ? reflux_of(a, g) : -1;
     __syncthreads();
-    float u[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    float u[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, r[5];
     if (t < 8 * s.nl) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) u[v] = a.U[v * a.S + g];
     }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) r[v] = pending(a, v, rs);
     if (leaf) {
-      const int rs = reflux_of(a, g);
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        float m[3], p[3];
+        const float *p = flux + v * TH + tid;
+        float m[3];
 #pragma unroll
-        for (int D = 0; D < 3; ++D) {
-          p[D] = plus[(5 * D + v) * nth + tid];
-          m[D] = from[D] >= 0 ? plus[(5 * D + v) * nth + from[D]] : from[D] == -1 ? 0.0f : minus[v * cap - 2 - from[D]];
-        }
-        u[v] = new_state(a, s, v, u[v], rs, pending(a, v, rs), flux_sum(m[0], p[0], m[1], p[1], m[2], p[2]));
-        a.U[v * a.S + g] = u[v];
+        for (int D = 0; D < 3; ++D) m[D] = from[D] < 0 ? 0.0f : flux[v * TH + from[D]];
+        u[v] = new_state(a, s, v, u[v], rs, r[v], flux_sum(m[0], p[0], m[1], p[5 * TH], m[2], p[10 * TH]));
       }
+#pragma unroll
+      for (int v = 0; v < 5; ++v) a.U[v * a.S + g] = u[v];
     }
     __syncthreads();  // the fluxes are read
     if (s.flags & kSegRestrict) {  // the warp's octs, a lane per (oct, variable)
 #pragma unroll
-      for (int v = 0; v < 5; ++v) plus[v * nth + tid] = u[v];
+      for (int v = 0; v < 5; ++v) flux[v * TH + tid] = u[v];
       __syncwarp();
       const int q = ((t - lane) >> 3) + (lane & 3), v = lane >> 2;
-      if (v < 5 && q < s.nl) restrict_oct(a, s, q, v, plus + v * nth + (tid - lane) + 8 * (lane & 3));
+      if (v < 5 && q < s.nl) restrict_oct(a, s, q, v, flux + v * TH + (tid - lane) + 8 * (lane & 3));
     }
   });
 }
