@@ -184,7 +184,9 @@ def kernel_traffic(info, levelmin, w, fused):
                   index (10 w + 4 B per real cell)
       both:
       prolong     7 sources in, 8 ghosts out        75 w per ghost oct
-      reflux_restrict  24 slots + R in/out per ghost oct (130 w), 8 children
+      reflux_restrict  (inside update, flux and the next prolong; launches of its
+                  own only where none follows)
+                  24 slots + R in/out per ghost oct (130 w), 8 children
                   in + father out per real oct above levelmin (45 w)
     """
     loc, real, ghost, fine = kernel_units(info, levelmin)
@@ -204,8 +206,8 @@ def kernel_traffic(info, levelmin, w, fused):
 # faces), and DRAM bytes per cell of the flux kernels, from one ncu capture
 # of the level-7 launch of the benchmark mesh (ncu: FP64 instruction counts,
 # dram__bytes_read.sum + dram__bytes_write.sum)
-FLUX_FP64_FLOPS_PER_CELL = 289.8
-FLUX_DRAM_BYTES_PER_CELL = {8: 272.7, 4: 125.8}
+FLUX_FP64_FLOPS_PER_CELL = 208.5
+FLUX_DRAM_BYTES_PER_CELL = {8: 272.6, 4: 124.1}
 
 
 def load_peaks():
@@ -695,9 +697,10 @@ def run_cic(n, reps, warmup, torch, peak_gbs, peak_src):
                "frac": round(alg / (k_ms * 1e-3) / 1e9 / peak_gbs, 4),
                "algorithmic_bytes": alg, "kernel_ms": round(k_ms, 4)}
         if prec == 8:
-            # bound by the FP64 pipe: FP64 thread instructions per particle
-            # counted by ncu (15 DMUL + 3 DFMA + 3.9 DADD on this set) against
-            # the pipe's issue rate; the SM clock is filled in after the run
+            # FP64 thread instructions per particle counted by ncu (0.93 DADD on this
+            # set; weights and products run on the integer pipes) against the pipe's
+            # issue rate; the SM clock is filled in after the run.  The deposit waits
+            # on its L2 atomics: the HBM view is beside it
             res["cic_atomic_roofline"] = {"bound": "alu", "unit": "G FP64 inst/s",
                                           "fp64_inst_per_particle": CIC_FP64_INST_PER_PARTICLE,
                                           "achieved": round(ps.np * CIC_FP64_INST_PER_PARTICLE
@@ -736,7 +739,7 @@ def run_cic_levels(timed, torch, st):
     return out
 
 
-CIC_FP64_INST_PER_PARTICLE = 21.9
+CIC_FP64_INST_PER_PARTICLE = 0.93
 
 
 def cic_alu_peak(cic, sm_mhz):

@@ -531,7 +531,10 @@ __device__ __forceinline__ void load_side(const StepArgs<float> &a, int o, int D
 // is the same number for both cells of a pair, so the pair's lanes each form it
 // for half of the variables and exchange it (24 differences per cell instead
 // of 30, and 15 loads instead of 30).  Bound by the FP64 pipe: 49 operations
-// per cell, 72 with every difference and product on it.
+// per cell, 72 with every difference and product on it.  Level 7 of the Sedov blast
+// 196 us (87 % of the FP64 pipe; 281 with 72 operations); all indices and loads come
+// first: waiting per axis, a coarse step of the 3-6 random mesh takes 208 us of it
+// instead of 140.
 __device__ __forceinline__ double shfl_xor_f64(unsigned mask, double x, int lanes) {
   const int lo = __shfl_xor_sync(mask, __double2loint(x), lanes), hi = __shfl_xor_sync(mask, __double2hiint(x), lanes);
   return __hiloint2double(hi, lo);
@@ -690,8 +693,8 @@ __device__ __forceinline__ void hllc(double rl, double ul, double al, double bl,
 // overflows, and the operands of mul (densities, pressures, wave speeds) are
 // normal with normal products.  Others take the FP64 pipe, with the same bits.
 // Level 7 of the Sedov blast (2.1 M cells): 780 us with all products on the
-// FP64 pipe, 497 us with them on the integer pipes (FP64 pipe 79 %, issue slots
-// 44 % busy).
+// FP64 pipe, 497 us with them on the integer pipes, 451 us with a block per tile and
+// axis (k_flux; FP64 pipe 87 %, issue slots 50 % busy).
 __device__ __forceinline__ void hllc_axis(int D, const double (&qL)[5], const double (&qR)[5], double g, double igm1,
                                           double (&F)[5]) {
   const bool x = D == 0, z = D == 2;
