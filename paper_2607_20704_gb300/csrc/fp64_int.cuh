@@ -58,34 +58,30 @@ __host__ __device__ __forceinline__ uint64_t mul_bits(uint64_t x, uint64_t y) {
   return (uint64_t(hi) << 32) | m;
 }
 
-// Sum of six doubles (bit k of NEG: the k-th is subtracted), rounded once, on the
-// integer pipes: the mantissas, shifted to the largest exponent with 7 bits below
-// its last place, add up in 64 bits (some 120 instructions; 5 additions hold the
-// FP64 pipe for 80 cycles of an SM).  Each term loses less than 2^-7 units in the
-// last place of the largest, the sum is then rounded to the nearest double:
-// against the exact sum at most 0.05 of those units more than one rounding, where
-// a chain of five additions rounds five times.  As in the products, what lies below
-// the normal range is zero.  `ok`: false where an operand is infinite, NaN or too
-// large for the sum; the caller then adds them on the FP64 pipe.
-template <unsigned NEG>
-__host__ __device__ __forceinline__ uint64_t sum6_bits(const uint64_t (&x)[6], bool &ok) {
-  uint32_t top = 0;
+// a + b + c of doubles given as bit patterns, rounded once, on the integer pipes: the
+// mantissas, shifted to the largest exponent with 8 bits below its last place, add up
+// in 64 bits.  Each term loses less than 2^-8 units in the last place of the largest;
+// a rounded addition loses up to half a unit of its result, and two are saved.  `ok`:
+// false where an operand is infinite, NaN or too large for the sum, or the result lies
+// below the normal range; the caller then adds on the FP64 pipe.
+__host__ __device__ __forceinline__ uint64_t sum3_bits(const uint64_t (&x)[3], bool &ok) {
+  constexpr uint32_t one = 1u << 20;  // one step of the exponent in a double's upper half
+  uint32_t e[3], top = one;           // (subnormal numbers have the smallest normal exponent)
+  uint64_t m[3], sum = 0;
 #pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    const uint32_t e = uint32_t(x[k] >> 32) & 0x7FF00000u;
-    top = e > top ? e : top;
+  for (int k = 0; k < 3; ++k) {
+    const uint32_t field = uint32_t(x[k] >> 32) & 0x7FF00000u;
+    m[k] = ((x[k] & 0xFFFFFFFFFFFFFull) | (field ? uint64_t(1) << 52 : 0)) << 8;
+    e[k] = field ? field : one;
+    top = e[k] > top ? e[k] : top;
   }
-  ok = top < (2042u << 20);
-  uint64_t sum = 0;
 #pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    const uint32_t h = uint32_t(x[k] >> 32), e = h & 0x7FF00000u;
-    const uint64_t m = e ? ((x[k] & 0xFFFFFFFFFFFFFull) | (uint64_t(1) << 52)) << 7 : 0;
-    const uint32_t d = (top - e) >> 20;
-    const uint64_t t = m >> (d < 63 ? d : 63);
-    const bool minus = (h >> 31) != ((NEG >> k) & 1u);
-    sum = minus ? sum - t : sum + t;
+  for (int k = 0; k < 3; ++k) {
+    const uint32_t d = (top - e[k]) >> 20;
+    const uint64_t t = m[k] >> (d < 63 ? d : 63);
+    sum = x[k] >> 63 ? sum - t : sum + t;
   }
+  ok = top < 2042u * one;
   const uint64_t neg = sum >> 63, a = neg ? 0 - sum : sum;
   if (a == 0) return 0;
 #ifdef __CUDA_ARCH__
@@ -95,8 +91,9 @@ __host__ __device__ __forceinline__ uint64_t sum6_bits(const uint64_t (&x)[6], b
 #endif
   const uint64_t n = a << z;
   const uint64_t r = (n >> 11) + ((n >> 10) & 1);
-  const int e = int(top >> 20) + 3 - z;  // of the sum, less one (the mantissa's leading bit adds it)
-  return e < 0 ? 0 : (neg << 63) | ((uint64_t(e) << 52) + r);
+  const int es = int(top >> 20) + 2 - z;  // of the sum, less one (the mantissa's leading bit adds it)
+  ok = ok && es >= 0;
+  return (neg << 63) | ((uint64_t(uint32_t(es)) << 52) + r);
 }
 
 #ifndef FP64_INT_HOST
@@ -117,21 +114,14 @@ __device__ __forceinline__ double mul_fp64_0(double x, double y) {
   return normal_or_zero(__dmul_rn(normal_or_zero(x), normal_or_zero(y)));
 }
 
-// not inlined: both sums would be formed and one chosen, five FP64 issues each time
-// (Sedov 7-10, update per coarse step: 450 instead of 359 us)
-__device__ __noinline__ double sum6_fp64(double a, double b, double c, double d, double e, double f) {
-  return __dadd_rn(__dadd_rn(__dadd_rn(a, b), __dadd_rn(c, d)), __dadd_rn(e, f));
-}
-template <unsigned NEG>
-__device__ __forceinline__ double sum6_int(double a, double b, double c, double d, double e, double f) {
-  const uint64_t x[6] = {uint64_t(__double_as_longlong(a)), uint64_t(__double_as_longlong(b)),
-                         uint64_t(__double_as_longlong(c)), uint64_t(__double_as_longlong(d)),
-                         uint64_t(__double_as_longlong(e)), uint64_t(__double_as_longlong(f))};
+// not inlined: both sums would be formed and one chosen
+__device__ __noinline__ double sum3_fp64(double a, double b, double c) { return __dadd_rn(__dadd_rn(a, b), c); }
+__device__ __forceinline__ double sum3_int(double a, double b, double c) {
+  const uint64_t x[3] = {uint64_t(__double_as_longlong(a)), uint64_t(__double_as_longlong(b)),
+                         uint64_t(__double_as_longlong(c))};
   bool ok;
-  const uint64_t s = sum6_bits<NEG>(x, ok);
-  if (ok) return __longlong_as_double((long long)s);
-  return sum6_fp64(NEG & 1 ? -a : a, NEG & 2 ? -b : b, NEG & 4 ? -c : c, NEG & 8 ? -d : d, NEG & 16 ? -e : e,
-                   NEG & 32 ? -f : f);
+  const uint64_t s = sum3_bits(x, ok);
+  return ok ? __longlong_as_double((long long)s) : sum3_fp64(a, b, c);
 }
 
 // x in [2^-E, 2^E)

@@ -819,11 +819,14 @@ __global__ void k_flux(StepArgs<double> a) {
   }
 }
 
-// sum over the axes of F(minus face) - F(plus face) of one variable; FP64 on the
-// integer pipes (five additions hold the FP64 pipe for 80 cycles of an SM), rounded
-// once
+// sum over the axes of F(minus face) - F(plus face) of one variable.  FP64: the three
+// differences on the FP64 pipe, which are exact where leading bits cancel (a pressure
+// that is nearly the same on both sides must not take bits from a small difference
+// along another axis), their sum on the integer pipes.  Sedov 7-10 / clustered 6-9, us
+// of updates per coarse step: 385 / 256; all five additions on the FP64 pipe 478 / 397,
+// none of them 405 / 258.
 __device__ __forceinline__ double flux_sum(double xm, double xp, double ym, double yp, double zm, double zp) {
-  return sum6_int<0x2A>(xm, xp, ym, yp, zm, zp);
+  return sum3_int(__dadd_rn(xm, -xp), __dadd_rn(ym, -yp), __dadd_rn(zm, -zp));
 }
 __device__ __forceinline__ float flux_sum(float xm, float xp, float ym, float yp, float zm, float zp) {
   return ((xm - xp) + (ym - yp)) + (zm - zp);
@@ -831,7 +834,7 @@ __device__ __forceinline__ float flux_sum(float xm, float xp, float ym, float yp
 
 // variable v of the pending reflux R in slot rs (-1: none).  Loaded with the fluxes,
 // before their sum: after it the load's latency comes on top (clustered 6-9, update
-// per coarse step: 439 instead of 253 us)
+// per coarse step: 439 instead of 256 us)
 template <class T>
 __device__ __forceinline__ T pending(const StepArgs<T> &a, int v, int rs) {
   return rs >= 0 ? a.Rc[v * int64_t(a.NC) + rs] : T(0);
@@ -874,10 +877,9 @@ __device__ __forceinline__ void restrict_oct(const StepArgs<T> &a, const SegCtx<
 // They touch disjoint data: the level's cells, the coarser level's split cells,
 // the pending reflux of its leaf cells.
 
-// FP64, a list that fills the GPU: a thread per cell, one variable after the other.
-// Sedov 7-10 / clustered 6-9, us per coarse step: 359 / 253; the sums on the FP64
-// pipe 481 / 385, the bound of that form.  The loads of the next variable ahead of
-// the sum: 371 / 256; at 40 registers 369 / 269.
+// FP64, a list that fills the GPU: a thread per cell, one variable after the other
+// (figures at flux_sum).  The loads of the next variable ahead of the sum, or 40
+// registers for more warps, gain nothing (3 % and more slower).
 // domain: 8 nl, + 5 ncl (if kSegReflux)
 __global__ void __launch_bounds__(512, 2) k_update(StepArgs<double> a) {
   extern __shared__ double update_smem[];  // the block's new states [5][threads]

@@ -1,6 +1,7 @@
 """FP64 arithmetic on the integer pipes (``csrc/fp64_int.cuh``) on the CPU (the
 header compiled for the host): products with the same bits as the native product
-for normal operands with a normal product; sums of six against the exact sum."""
+for normal operands with a normal product; the sum of three flux differences against
+the exact one."""
 import ctypes
 import math
 import os
@@ -13,6 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(os.path.dirname(HERE), "paper_2607_20704_gb300", "csrc")
 SRC = """
 #include <cstdint>
+#include <cstring>
 #define __host__
 #define __device__
 #define __forceinline__ inline
@@ -24,11 +26,16 @@ extern "C" void mul_many(const uint64_t *a, const uint64_t *b, uint64_t *c, long
 extern "C" void mul_many0(const uint64_t *a, const uint64_t *b, uint64_t *c, long n) {
   for (long i = 0; i < n; ++i) c[i] = amr::mul_bits<true>(a[i], b[i]);
 }
-extern "C" void sum_many(const uint64_t *a, uint64_t *c, unsigned char *ok, long n) {
+extern "C" void sum_many(const double *a, double *c, unsigned char *ok, long n) {
   for (long i = 0; i < n; ++i) {
-    const uint64_t x[6] = {a[6 * i], a[6 * i + 1], a[6 * i + 2], a[6 * i + 3], a[6 * i + 4], a[6 * i + 5]};
+    uint64_t x[3], s;
+    for (int k = 0; k < 3; ++k) {
+      const double d = a[6 * i + 2 * k] - a[6 * i + 2 * k + 1];
+      std::memcpy(&x[k], &d, 8);
+    }
     bool o;
-    c[i] = amr::sum6_bits<0x2A>(x, o);
+    s = amr::sum3_bits(x, o);
+    std::memcpy(&c[i], &s, 8);
     ok[i] = o;
   }
 }
@@ -95,8 +102,20 @@ def test_products_below_the_normal_range_are_zero(lib):
     assert np.array_equal(c[ok], want.view(np.uint64)[ok])
 
 
+def _check_sums(lib, a):
+    """The sum of the three (rounded) differences within half a unit in the last place
+    of the result and 3 2^-8 units of the largest difference: what three terms lose."""
+    n = len(a)
+    x, c, ok = a.view(np.float64), np.zeros(n), np.zeros(n, np.uint8)
+    lib.sum_many(_ptr(x), _ptr(c), _ptr(ok), ctypes.c_long(n))
+    assert ok.all()
+    d = x[:, ::2] - x[:, 1::2]
+    for r, t in zip(c, d):
+        assert abs(math.fsum([r, *-t])) <= 0.5 * math.ulp(r) + 3 * 2.0 ** -8 * math.ulp(abs(t).max()), (t, r)
+
+
 @pytest.mark.parametrize("spread", [0, 2, 30, 60, 500])
-def test_sums_of_six_round_once(lib, spread):
+def test_sums_of_three_differences_round_once(lib, spread):
     rng = np.random.default_rng(5 + spread)
     n = 20000
     a = _bits(rng, 6 * n, spread).reshape(n, 6)
@@ -104,22 +123,32 @@ def test_sums_of_six_round_once(lib, spread):
     a[1::3, 3] = a[1::3, 2] ^ np.uint64(1)             # nearly
     a[::5, 4:] &= np.uint64(1 << 63)                   # zeros of either sign
     a[:9] &= np.uint64(1 << 63)
-    x, c, ok = a.view(np.float64), np.zeros(n, np.uint64), np.zeros(n, np.uint8)
-    lib.sum_many(_ptr(a), _ptr(c), _ptr(ok), ctypes.c_long(n))
-    assert ok.all()
-    got = c.view(np.float64)
-    for r, t in zip(got, x * [1, -1, 1, -1, 1, -1]):
-        # five terms lose less than 2^-7 units in the last place of the largest each
-        assert abs(math.fsum([r, *-t])) <= 0.5 * math.ulp(r) + 5 * 2.0 ** -7 * math.ulp(abs(t).max())
+    _check_sums(lib, a)
+
+
+@pytest.mark.parametrize("pair", [0, 2, 4])
+def test_a_large_pair_takes_nothing_from_a_small_difference(lib, pair):
+    """A flux that is (nearly) the same on both faces of one axis beside fluxes 2^40 to
+    2^400 times smaller along the others: the small difference is what moves the cell."""
+    rng = np.random.default_rng(11 + pair)
+    n = 20000
+    a = _bits(rng, 6 * n, 20).reshape(n, 6)
+    a[:, pair] += rng.integers(60, 400, n).astype(np.uint64) << np.uint64(52)
+    a[:, pair + 1] = a[:, pair]
+    a[::7, pair + 1] += np.uint64(1)                   # one unit in the last place apart
+    near = (pair + 2) % 6
+    a[1::2, near + 1] = a[1::2, near] + rng.integers(0, 1 << 20, len(a[1::2])).astype(np.uint64)
+    _check_sums(lib, a)
 
 
 def test_sums_at_the_ends_of_the_range(lib):
-    a = np.zeros((7, 6))
+    a = np.zeros((9, 6))
     a[0, 2], a[1, 5], a[2, 0] = np.inf, np.nan, 2.0 ** 1020  # refused
-    a[3, 1] = 5e-324                                         # below the normal range: zero
-    a[4, 3], a[5, 2] = 2.0 ** -1022, -(2.0 ** -960)          # exact
-    a[6, :] = 2.0 ** 1018
-    c, ok = np.zeros(7, np.uint64), np.zeros(7, np.uint8)
-    lib.sum_many(_ptr(a), _ptr(c), _ptr(ok), ctypes.c_long(7))
-    assert ok.tolist() == [0, 0, 0, 1, 1, 1, 1]
-    assert c.view(np.float64)[3:].tolist() == [0.0, -(2.0 ** -1022), -(2.0 ** -960), 0.0]
+    a[3, 1], a[4, 2:4] = 5e-324, (2.0 ** -1022, 5e-324)      # a result below the normal range: refused
+    a[5, 3], a[6, 2] = 2.0 ** -1022, -(2.0 ** -960)          # exact
+    a[7, :] = 2.0 ** 1018
+    a[8, :] = 5e-324
+    c, ok = np.zeros(9), np.zeros(9, np.uint8)
+    lib.sum_many(_ptr(a), _ptr(c), _ptr(ok), ctypes.c_long(9))
+    assert ok.tolist() == [0, 0, 0, 0, 0, 1, 1, 1, 1]
+    assert c[5:].tolist() == [-(2.0 ** -1022), -(2.0 ** -960), 0.0, 0.0]

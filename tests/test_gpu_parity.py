@@ -366,6 +366,21 @@ def test_fp32_runs_repeat_bit_for_bit():
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("amplitude", [1e-6, 1e-9, 1e-12])
+@pytest.mark.parametrize("level,ns,planar", [(5, 0, 0), (6, 0, 0), (5, 2, 0), (5, 2, 1)])
+def test_weak_shear_beside_equal_pressures(level, ns, planar, amplitude):
+    """A shear u(y) far below the sound speed: the pressure fluxes along x cancel, and
+    what changes the x-momentum is a small difference along y.  Level 5 takes the
+    update of short lists, level 6 that of long ones, the others the fused kernels."""
+    prob = inputs.uniform_grid(level, lambda x, y, z: (1.0 + 0 * x, amplitude * np.sin(2 * np.pi * y), 0.3 + 0 * x,
+                                                       0 * x, 1.0 + 0 * x))
+    g, o = pair(prob, gpu_kw=dict(tile=128, schedule=0, nsubgrid=ns, planar=planar))
+    dt = o.cfl_dt()
+    g.step_level(level, dt)
+    o.step_level(level, dt)
+    compare_all(g, o, 1e-12)
+
+
 def _deepest():
     # levels 2..15 (the deepest a handle holds: 4-bit level, 14-bit
     # coordinates), 27 octs per level around an off-centre point
