@@ -182,11 +182,14 @@ def test_repack_rejects_bad_arguments_and_keeps_the_handle():
     b.close()
 
 
-@pytest.mark.parametrize("precision,tile", [(8, 64), (4, 64), (4, 512)])
+@pytest.mark.parametrize("precision,tile", [(8, 64), (8, 512), (4, 64), (4, 512)])
 def test_short_and_long_lists_step_alike(precision, tile):
-    """A mesh alone has levels of at most 15 thousand local cells (more threads per
-    cell); 24 copies of it in one batch share lists of some 300 thousand (the
-    kernels that fill the GPU): the same states, reflux and restriction included."""
+    """A mesh alone has levels of at most 15 thousand local cells, each a list of one
+    segment (which its launch carries as an argument); 24 copies of it in one batch
+    share lists of 24 segments and some 300 thousand cells, with tiles of other members
+    beside their own.  In FP64 the first take the update with a thread per (cell,
+    variable) and the second the one with a thread per cell; FP32 has one kernel for
+    both.  The same states, reflux and restriction included."""
     from paper_2607_20704_gb300 import amr
     pr = inputs.random_mesh(3, 6, seed=5)
     kw = dict(precision=precision, nsubgrid=0, tile=tile, schedule=0)
