@@ -1105,11 +1105,12 @@ __global__ void k_restrict(StepArgs<T> a) {
 
 // ---------------------------------------------------------------------------
 // CFL time step: per (member, level) max of sum_d (|u_d| + c) over leaf cells
-// (cell speeds in the state's precision, the maximum and dt in FP64): block
-// reduction of each tile (warp shuffles, then shared memory), one integer
-// atomicMax per tile on the bit pattern (non-negative doubles order like their
-// bits); then one thread per member computes its dt.
+// (cell speeds in the state's precision, the maximum and dt in FP64), by integer
+// atomicMax on the bit pattern (non-negative doubles order like their bits): FP32
+// once per block and segment, FP64 once per warp that formed a speed; then one
+// thread per member computes its dt.
 // ---------------------------------------------------------------------------
+// the block's maximum over a segment: warp shuffles, then shared memory
 template <class T>
 __device__ __forceinline__ void cfl_flush(const CflArgs &a, double s, int seg, double *wmax) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
