@@ -894,13 +894,14 @@ static void run_prolong(amr_mesh *h, StepArgs<T> a, const SegList &L, const SegL
   launch(h, K_PROLONG, k_prolong<T>, dim3(unsigned(grid)), dim3(unsigned(h->tile_size)), a, p);
 }
 
-// FP64: up to this many local cells a list does not fill the GPU, and the update
-// lasts as long as its chain of loads and arithmetic: it takes k_update_small, with a
-// thread per (cell, variable).  Times of a step, that kernel against the other: levels
-// of 2-15 thousand cells (random mesh 3-6) 0.295 against 0.334 ms, of 15-50 thousand
-// (Sedov 6-9) 0.486 against 0.511 ms, of 25-72 thousand (Sod 5-6) 107 against 109 us;
-// with lists of up to 131 thousand in it, clustered 6-9, 1.136 against 1.125 ms; a
-// level of 262 thousand 162 against 140 us.
+// FP64: up to this many local cells (431 per SM) the update lasts as long as its chain
+// of loads and arithmetic, and takes k_update_small, with a thread per (cell, variable);
+// beyond, the pipes are busy enough with a thread per cell.  Step times, that kernel
+// against the other: 512 cells 28.8 against 32.8 us; levels of 2-15 thousand (random
+// mesh 3-6) 0.295 against 0.330 ms; of 15-50 thousand (Sedov 6-9) 0.492 against 0.512
+// ms; of 25-72 thousand (Sod 5-6) equal.  With lists of up to 131 thousand in it,
+// clustered 6-9 takes 1.149 instead of 1.134 ms; with every list, a level of 262
+// thousand 150 instead of 146 us, Sedov 7-10 2.19 instead of 2.03 ms.
 constexpr int kSmallList = 65536;
 
 template <class T>
