@@ -204,10 +204,10 @@ def kernel_traffic(info, levelmin, w, fused):
 
 # FP64 flops (2 per FMA) per real cell of the FP64 flux kernel (three HLLC
 # faces), and DRAM bytes per cell of the flux kernels, from one ncu capture
-# of the level-7 launch of the benchmark mesh (ncu: FP64 instruction counts,
+# of the level-7 launch of a coarse step of the benchmark mesh (ncu: FP64 instruction counts,
 # dram__bytes_read.sum + dram__bytes_write.sum)
-FLUX_FP64_FLOPS_PER_CELL = 208.5
-FLUX_DRAM_BYTES_PER_CELL = {8: 272.6, 4: 124.1}
+FLUX_FP64_FLOPS_PER_CELL = 196.5
+FLUX_DRAM_BYTES_PER_CELL = {8: 272.4, 4: 124.0}
 
 
 def load_peaks():

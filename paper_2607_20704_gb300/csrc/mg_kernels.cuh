@@ -12,8 +12,8 @@
 // The base level lives in the mesh's oct order; the solver works on dense
 // arrays [x + n (y + n z)] of every multigrid level (unit-stride x, so every
 // stencil access is coalesced), gathered from and scattered back to the octs.
-// On GB300 the FP64 pipe bounds these stencils on the large grids (7 FP64
-// operations per smoothed cell against 16 bytes of traffic) and the launches on
+// On GB300 the FP64 pipe bounds these stencils on the large grids (6 FP64
+// instructions per smoothed cell against 16 bytes of traffic) and the launches on
 // the small ones; no step divides: the Gauss-Seidel update multiplies by the
 // rounded 1/6 where the operator divides by 6 (the two differ by at most a few
 // units in the last place per update; the product runs on the integer pipes),
@@ -114,7 +114,7 @@ __global__ void k_mg_smooth(int b, double dx2, const double *__restrict__ f, dou
 // coarse source = mean of the 8 children's residuals; coarse correction = 0.
 // Three of a child's neighbours lie in the block of 8 and cancel against half
 // of its diagonal when the residuals are summed: the sum needs, per child, its
-// three outer neighbours less 3 p (39 FP64 operations per block, 72 with eight
+// three outer neighbours less 3 p (42 FP64 operations per block, 72 with eight
 // residuals).
 __device__ __forceinline__ double mg_block_residual(int n, double inv_dx2, const double *__restrict__ f,
                                                     const double *__restrict__ p, int X, int Y, int Z) {
