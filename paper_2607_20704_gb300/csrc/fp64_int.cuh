@@ -62,8 +62,10 @@ __host__ __device__ __forceinline__ uint64_t mul_bits(uint64_t x, uint64_t y) {
 // mantissas, shifted to the largest exponent with 8 bits below its last place, add up
 // in 64 bits.  Each term loses less than 2^-8 units in the last place of the largest;
 // a rounded addition loses up to half a unit of its result, and two are saved.  `ok`:
-// false where an operand is infinite, NaN or too large for the sum, or the result lies
-// below the normal range; the caller then adds on the FP64 pipe.
+// false where an operand is infinite, NaN or too large for the sum, where the result
+// lies below the normal range, or where the terms cancel to less than 2^-12 of the
+// largest (what they lost is then more than 2^-46 of the result, and two of them may
+// cancel exactly beside a small third); the caller then adds on the FP64 pipe.
 __host__ __device__ __forceinline__ uint64_t sum3_bits(const uint64_t (&x)[3], bool &ok) {
   constexpr uint32_t one = 1u << 20;  // one step of the exponent in a double's upper half
   uint32_t e[3], top = one;           // (subnormal numbers have the smallest normal exponent)
@@ -81,8 +83,8 @@ __host__ __device__ __forceinline__ uint64_t sum3_bits(const uint64_t (&x)[3], b
     const uint64_t t = m[k] >> (d < 63 ? d : 63);
     sum = x[k] >> 63 ? sum - t : sum + t;
   }
-  ok = top < 2042u * one;
   const uint64_t neg = sum >> 63, a = neg ? 0 - sum : sum;
+  ok = top < 2042u * one && (a >> 48 || (m[0] | m[1] | m[2]) == 0);  // the largest is 2^60 and more
   if (a == 0) return 0;
 #ifdef __CUDA_ARCH__
   const int z = __clzll((long long)a);

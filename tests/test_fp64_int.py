@@ -102,16 +102,23 @@ def test_products_below_the_normal_range_are_zero(lib):
     assert np.array_equal(c[ok], want.view(np.uint64)[ok])
 
 
-def _check_sums(lib, a):
+def _check_sums(lib, a, most):
     """The sum of the three (rounded) differences within half a unit in the last place
-    of the result and 3 2^-8 units of the largest difference: what three terms lose."""
+    of the result and 3 2^-8 units of the largest difference: what three terms lose.
+    Refused only where they cancel to less than 2^-12 of the largest (2^-11 for the
+    terms' own loss and the largest mantissa); `most`: the share that may."""
     n = len(a)
     x, c, ok = a.view(np.float64), np.zeros(n), np.zeros(n, np.uint8)
     lib.sum_many(_ptr(x), _ptr(c), _ptr(ok), ctypes.c_long(n))
-    assert ok.all()
     d = x[:, ::2] - x[:, 1::2]
-    for r, t in zip(c, d):
-        assert abs(math.fsum([r, *-t])) <= 0.5 * math.ulp(r) + 3 * 2.0 ** -8 * math.ulp(abs(t).max()), (t, r)
+    assert np.count_nonzero(ok == 0) <= most * n
+    for r, o, t in zip(c, ok, d):
+        exact, big = math.fsum(t), abs(t).max()
+        if o:
+            assert abs(math.fsum([r, *-t])) <= 0.5 * math.ulp(r) + 3 * 2.0 ** -8 * math.ulp(big), (t, r)
+            assert abs(math.fsum([r, *-t])) <= 2.0 ** -45 * abs(exact), (t, r)
+        else:
+            assert big > 0 and abs(exact) <= 2.0 ** -11 * big, (t, r)
 
 
 @pytest.mark.parametrize("spread", [0, 2, 30, 60, 500])
@@ -123,7 +130,7 @@ def test_sums_of_three_differences_round_once(lib, spread):
     a[1::3, 3] = a[1::3, 2] ^ np.uint64(1)             # nearly
     a[::5, 4:] &= np.uint64(1 << 63)                   # zeros of either sign
     a[:9] &= np.uint64(1 << 63)
-    _check_sums(lib, a)
+    _check_sums(lib, a, 0.02)
 
 
 @pytest.mark.parametrize("pair", [0, 2, 4])
@@ -138,7 +145,20 @@ def test_a_large_pair_takes_nothing_from_a_small_difference(lib, pair):
     a[::7, pair + 1] += np.uint64(1)                   # one unit in the last place apart
     near = (pair + 2) % 6
     a[1::2, near + 1] = a[1::2, near] + rng.integers(0, 1 << 20, len(a[1::2])).astype(np.uint64)
-    _check_sums(lib, a)
+    _check_sums(lib, a, 0.02)
+
+
+@pytest.mark.parametrize("axes", [(0, 2), (0, 4), (2, 4)])
+def test_differences_that_cancel_are_left_to_the_fp64_pipe(lib, axes):
+    """Two axes whose differences are (nearly) opposite beside a small third."""
+    rng = np.random.default_rng(17 + sum(axes))
+    n = 20000
+    a = _bits(rng, 6 * n, 20).reshape(n, 6)
+    p, q = axes
+    a[:, [p, p + 1]] += (rng.integers(42, 400, n).astype(np.uint64) << np.uint64(52))[:, None]
+    a[:, q], a[:, q + 1] = a[:, p + 1], a[:, p]
+    a[::7, q] ^= np.uint64(1)
+    _check_sums(lib, a, 1.0)
 
 
 def test_sums_at_the_ends_of_the_range(lib):
